@@ -344,14 +344,14 @@ int rvh_get_stats(rvh_ctx* ctx, rvh_stats* out);
 int rvh_set_schedule(rvh_ctx* ctx, int32_t points_per_warp, int32_t hyps_per_lane);
 
 /* Staged scoring with exact pruning (default on): the scoring pass of a
- * cluster of at least 512 points whose rows fit shared memory (the
+ * cluster of at least 256 points whose rows fit shared memory (the
  * lanes-over-trials schedule, points_per_warp 1) runs in stages, the first
- * of 128 points and each later one half as long again; after the first,
- * the trial with the highest partial count is
- * counted exactly and leads, and after each stage a trial whose partial
- * count plus the points still to come cannot beat the lead's (count, lower
- * index) key is dropped.  Counts only grow by one per point and the exact
- * count never exceeds the upper-bound count, so no dropped trial can win:
+ * two of 128 points and each later one twice as long.  After the first,
+ * the trial with the highest partial count leads: it is counted over every
+ * point, and its residuals bound how many of the points still to come any
+ * other trial can hold.  After each stage a trial whose partial count plus
+ * that bound cannot beat the lead's (count, lower index) key is dropped.
+ * No exact count exceeds its bound, so no dropped trial can win:
  * every output equals the unpruned pass's (the winner of Sec. III-A over
  * all trials of Alg. 1), with fewer (trial, point) evaluations
  * (rvh_stats.pairs_scored).  enabled: 1 on, 0 off. */

@@ -32,51 +32,16 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
-__device__ __forceinline__ int block_max_int(int v, int* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+// Block reductions.  Each warp reduces with one redux instruction per 32-bit
+// word, its lane 0 leaves the result in red, and after one barrier every
+// thread combines the kWarps results.  There is no barrier in front: red has
+// to be an array that no thread can still be reading from an earlier use,
+// i.e. at least one other barrier lies between two uses of it.
+__device__ __forceinline__ unsigned long long block_best(int count, int h, unsigned long long* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  int r = red[0];
-#pragma unroll
-  for (int w = 1; w < kWarps; ++w) r = max(r, red[w]);
-  return r;
-}
-
-__device__ __forceinline__ int block_min_int(int v, int* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  int r = red[0];
-#pragma unroll
-  for (int w = 1; w < kWarps; ++w) r = min(r, red[w]);
-  return r;
-}
-
-__device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long v, unsigned long long* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  unsigned long long r = 0;
-#pragma unroll
-  for (int w = 0; w < kWarps; ++w) r += red[w];
-  return r;
-}
-
-__device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v, unsigned long long* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
+  const int c = __reduce_max_sync(0xffffffffu, count);
+  const int hm = __reduce_min_sync(0xffffffffu, count == c ? h : 0x7fffffff);
+  if (lane == 0) red[warp] = c >= 0 ? best_key(c, hm) : 0ull;
   __syncthreads();
   unsigned long long r = red[0];
 #pragma unroll
@@ -84,17 +49,29 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v
   return r;
 }
 
-__device__ __forceinline__ float block_max_float(float v, float* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+// sums of a and b (each below 2^31 over the block), a in the low word
+__device__ __forceinline__ unsigned long long block_sum2(unsigned a, unsigned b, unsigned long long* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  a = __reduce_add_sync(0xffffffffu, a);
+  b = __reduce_add_sync(0xffffffffu, b);
+  if (lane == 0) red[warp] = (unsigned long long)b << 32 | a;
   __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  float r = red[0];
+  unsigned long long r = 0;
 #pragma unroll
-  for (int w = 1; w < kWarps; ++w) r = fmaxf(r, red[w]);
+  for (int w = 0; w < kWarps; ++w) r += red[w];
   return r;
+}
+
+// maximum of non-negative floats (their bit patterns order like integers)
+__device__ __forceinline__ float block_max_float(float v, int* red) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m = __reduce_max_sync(0xffffffffu, __float_as_int(v));
+  if (lane == 0) red[warp] = m;
+  __syncthreads();
+  int r = red[0];
+#pragma unroll
+  for (int w = 1; w < kWarps; ++w) r = max(r, red[w]);
+  return __int_as_float(r);
 }
 
 // ---- a4: upper-bound counts U_h = #{|r32| <= thi_h} (the hot loop) -----------------
@@ -221,17 +198,107 @@ __device__ bool hyp_f64(const FrameDesc& a, const RS& R, int ci, int h, int N, d
   return solve_f64<DIM>(r0, r1, r2, w, a.eps, v, nullptr);
 }
 
+// ---- what the lead's residuals say about every other trial --------------------------
+// The lead L (a trial with a high exact count) has a residual
+// r_L(j) = w_j - a_j.v_L at every point, and trial h's is r_L(j) - a_j.d with
+// d = v_h - v_L.  So h can only hold
+//   - points with |r_L| <= tau + max|a.d|, of those the lead does not hold, and
+//   - points with |a.d| <= tau + |r_L| <= 2 tau, of those it does: with
+//     t = a1 / a0 (the tangent of the azimuth) that is an interval of t,
+//     |d0 + d1 t| <= (2 tau + max|a2 d2|) / min a0.
+// Two histograms over the points still to be scored -- the excess |r_L| -
+// thi of the points outside the lead, a quarter octave per bin, and t of the
+// points inside, evenly over the cluster's range -- turn both into counts
+// per trial, which replace "every point still to come" in the pruning test.
+// Everything is rounded so that the counts only err upwards: bins are taken
+// by the same monotone FP32 expressions on both sides, and the band
+// half-widths of both trials (which bound the FP32 residuals' and
+// velocities' errors) are added to the thresholds.
+constexpr int kExcessBins = 64, kTanBins = 32;
+constexpr int kExcessBase = 119 << 2;  // bin 0: an excess below 2^-8 m/s
+
+__device__ __forceinline__ int excess_bin(float x) {
+  return min(max((__float_as_int(x) >> 21) - kExcessBase, 0), kExcessBins - 1);
+}
+
+// The cluster's directions a: range of t = a1 / a0, 1 / min a0 and max|a2|;
+// tan_ok = 0 (some a0 not safely positive, or rows that are no directions)
+// leaves the interval test out.
+struct DirRange {
+  float t0, tinv, tabs, a0inv, zmax;
+  int tan_ok;
+};
+
+__device__ __forceinline__ int tan_bin(const DirRange& g, float t) {
+  return min(max(__float2int_rd((t - g.t0) * g.tinv), 0), kTanBins - 1);
+}
+
+// floats as integers of the same order, and back
+__device__ __forceinline__ int float_order(float f) {
+  const int i = __float_as_int(f);
+  return i ^ (i >> 31 & 0x7fffffff);
+}
+__device__ __forceinline__ float order_float(int i) { return __int_as_float(i ^ (i >> 31 & 0x7fffffff)); }
+
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Upper bound of a normal record's band half-width.
+__device__ __forceinline__ float record_band(float4 hy, float tau_hi, bool line) {
+  return line ? 0x1p-21f * (1.0f + fabsf(hy.x) + fabsf(hy.y) + hy.w) : fmaxf(hy.w - tau_hi, 0.0f) + 0x1p-20f * hy.w;
+}
+
+// The certain-inlier threshold of a record: |r32| <= tlo is an inlier.  Its
+// upper threshold thi is tau + b rounded up, so thi - tau bounds the band
+// half-width b; for the line model record_band does, and both thresholds
+// are b away from T distd.
+__device__ __forceinline__ float record_tlo(float4 hy, TauPair tau, bool line) {
+  return line ? hy.w * (1.0f - 0x1p-20f) - 2.0f * record_band(hy, tau.hi, true)
+              : __fsub_rd(tau.lo, __fsub_ru(hy.w, tau.hi));
+}
+
+// Where a trial's points can lie, as bins: excess bins 0 .. out of the points
+// outside the lead, t bins lo .. hi - 1 of those inside.  Packed in one word.
+struct HoldRange {
+  uint32_t v;
+  __device__ __forceinline__ int out() const { return (int)(v & 255u); }
+  __device__ __forceinline__ int lo() const { return (int)(v >> 8 & 255u); }
+  __device__ __forceinline__ int hi() const { return (int)(v >> 16); }
+};
+
+template <int DIM>
+__device__ __forceinline__ HoldRange hold_range(const DirRange& g, float4 lead, float lead_band, float tau_hi,
+                                                bool line, float4 hy) {
+  const float dx = hy.x - lead.x, dy = hy.y - lead.y, dz = DIM == 3 ? hy.z - lead.z : 0.0f;
+  const float ax = fabsf(dx), ay = fabsf(dy), az = DIM == 3 ? g.zmax * fabsf(dz) : 0.0f;
+  const float slack = 2.0f * (record_band(hy, tau_hi, line) + lead_band) + 4e-6f * (ax + ay + fabsf(dz));
+  // max|a.d|: unit directions, or (x, 1) with x in [0, 1] for the line model
+  const float reach = line ? ax + ay : sqrt_approx(fmaf(dx, dx, dy * dy)) + az;
+  const uint32_t out = (uint32_t)excess_bin((hy.w + reach + slack) * 1.0001f - lead.w);
+  uint32_t lo = 0u, hi = kTanBins;
+  if (g.tan_ok) {
+    const float K = (hy.w + lead.w + slack + az) * g.a0inv * 1.0001f + 1e-5f * (ax + ay * g.tabs);
+    const float r = rcp_approx(dy);  // dy = 0: ends at +-inf, all of t or none of it
+    const float u = (-dx - K) * r, v = (K - dx) * r;
+    lo = (uint32_t)min(max(__float2int_rd((fminf(u, v) - g.t0) * g.tinv), 0), kTanBins);
+    hi = (uint32_t)max(min(__float2int_rd((fmaxf(u, v) - g.t0) * g.tinv), kTanBins - 1) + 1, (int)lo);
+  }
+  return HoldRange{out | lo << 8 | hi << 16};
+}
+
 struct ClusterShared {
   unsigned long long best;
-  float wmax;
   float4 win;      // winner's FP32 record
-  float win_tlo;
   int red_i[kWarps];
-  float red_f[kWarps];
+  int red_f[kWarps];
   double red_t[9];            // the normal-equation sums of the winner's inliers
   unsigned long long ctr[4];  // exact counts, band points, fp64 trials, refined trials
   unsigned long long clk[6];  // cycles per stage (thread 0's view of the CTA)
-  unsigned long long red_u[kWarps];
+  unsigned long long red_u[kWarps];  // block_best
+  unsigned long long red_v[kWarps];  // block_sum2
   double cv64[3];             // FP64 velocity of the trial being counted (when it has band points)
   double win_v64[3];          // FP64 velocity of the current winner (valid if win_has_v64)
   int win_has_v64;
@@ -247,6 +314,15 @@ struct ClusterShared {
   unsigned long long runs[2];  // trials run, pairs scored
   unsigned long long scored;   // (trial, point) pairs the scoring pass evaluated
   int nref;                   // 2D trials queued for refinement in the current chunk
+  DirRange dir;               // the cluster's directions (staged pass)
+  int red_d[4][kWarps];
+  // Points still to be scored when the lead was taken, by its residual:
+  // inside it, those below each bin of t; outside it, those up to each bin of
+  // the excess.  From stage 0 / 1 on and, in the second half, from 2 / 3 on,
+  // as 16-bit halves.
+  unsigned lead_in[2 * (kTanBins + 1)];
+  unsigned lead_out[2 * kExcessBins];
+  unsigned lead_cnt;          // the lead's certain points and band points
 };
 
 // Adaptive trial count: with `best` the best (count + 1, -index) key so far,
@@ -464,13 +540,13 @@ template <int DIM, typename RV, bool EXT>
 __device__ int exact_count_block(const FrameDesc& a, const RV rows, const Rows64<DIM>& R,
                                  int ci, int h, int N, float4 hy, float tlo, ClusterShared& cs, int* band) {
   const int tid = threadIdx.x;
-  unsigned long long lb = 0;  // L in the low word, B in the high word
+  unsigned in = 0, near = 0;
   for (int j = tid; j < N; j += kThreads) {
     const float r = fabsf(resid_f32<DIM>(rows.at(j), hy.x, hy.y, hy.z));
-    if (r <= tlo) lb += 1ull;
-    else if (!(r > hy.w)) lb += 1ull << 32;
+    if (r <= tlo) ++in;
+    else if (!(r > hy.w)) ++near;
   }
-  lb = block_sum_u64(lb, cs.red_u);
+  const unsigned long long lb = block_sum2(in, near, cs.red_v);
   const int L = (int)(lb & 0xFFFFFFFFull), B = (int)(lb >> 32);
   *band = B;
   if (B == 0) return L;
@@ -490,7 +566,7 @@ __device__ int exact_count_block(const FrameDesc& a, const RV rows, const Rows64
   }
   __syncthreads();
   const double v[3] = {cs.cv64[0], cs.cv64[1], cs.cv64[2]};
-  unsigned long long lbin = 0;
+  unsigned lbin = 0;
   auto cosine_band = [&]() {
     for (int j = tid; j < N; j += kThreads) {
       const float4 row = rows.at(j);
@@ -517,8 +593,7 @@ __device__ int exact_count_block(const FrameDesc& a, const RV rows, const Rows64
   } else {
     cosine_band();
   }
-  lbin = block_sum_u64(lbin, cs.red_u);
-  return L + (int)lbin;
+  return L + (int)block_sum2(lbin, 0u, cs.red_v);
 }
 
 template <int DIM>
@@ -779,24 +854,20 @@ __device__ __noinline__ int local_opt_rounds(const FrameDesc& a, const RV rows, 
   return n_in;
 }
 
-// Keeps, in order, the entries of S.list[0 .. n) (from_list) or the trials
-// 0 .. n - 1 for which keep(h) holds, writing them to S.list[0 ..); returns
-// how many.  Entries are read before any is written (compaction in place).
-// red: kWarps ints of shared memory.
-template <typename Keep>
-__device__ __forceinline__ int compact_list(const Smem& S, int n, bool from_list, Keep keep, int* red) {
+// Keeps, in order, the trials at positions 0 .. n - 1 of the staged pass's
+// list (list_trial) for which keep(h) holds, writing them to S.list[0 ..);
+// returns how many.  Entries are read before any is written (compaction in
+// place).  red: kWarps ints of shared memory.
+template <bool LISTED, typename Keep>
+__device__ __forceinline__ int prune_list(const Smem& S, int n, Keep keep, int* red) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int out = 0;
   for (int r0 = 0; r0 < n; r0 += 4 * kThreads) {
     int hv[4], c = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int i = r0 + 4 * tid + k;
-      int h = -1;
-      if (i < n) {
-        h = from_list ? (int)S.list[i] : i;
-        if (h == (int)kDropped || !keep(h)) h = -1;
-      }
+      int h = list_trial<LISTED>(S, n, r0 + 4 * tid + k);
+      if (h >= 0 && !keep(h)) h = -1;
       hv[k] = h;
       c += h >= 0 ? 1 : 0;
     }
@@ -824,55 +895,230 @@ __device__ __forceinline__ int compact_list(const Smem& S, int n, bool from_list
   return out;
 }
 
-// Drops the entries of S.list[0 .. n) (n <= 4 kThreads) for which keep(h)
-// fails: marked kDropped in place, and the list compacted (in order) only
-// when its groups of 128 would be fewer.  Returns the new list length
-// (marked entries included when it was not compacted).  red: kWarps ints.
-template <typename Keep>
-__device__ __forceinline__ int prune_list(const Smem& S, int n, Keep keep, int* red) {
+// ---- the staged scoring pass (a4 with exact pruning) ---------------------------------
+// Quads (4 points) of the first stage and of the next one; each later stage
+// is twice the one before.  Clusters of fewer than kStageMinPoints points
+// are scored in one pass.  What bounds the pass is the FP32 scoring of the
+// pairs that stay (8.6e12 pairs/s inside the kernel, 9.15e12 in isolation),
+// then the lead pass, the histograms' scans and the first pruning test,
+// together about 40 points' worth of scoring 1024 trials.  Measured, ms per
+// frame (dense2d / stress2d / dense3d): without the pass 0.292 / 0.846 /
+// 1.93; pruning by "every point still to come" instead of the lead's
+// residuals (72% / 100% / 66% of the pairs) 0.261 / 0.845 / 1.688; this pass
+// (42% / 59% / 38%) 0.221 / 0.787 / 1.480.  First stage of 64 / 96 / 128
+// points 0.229 / 0.224 / 0.221 (a longer one finds a better lead), threshold
+// of 192 instead of 256 points 0.223 / 0.802 / 1.495; a new lead after every
+// early stage evaluates fewer pairs (29%) but took 0.305 ms.
+constexpr int kStage0Quads = 32, kStage1Quads = 32;
+constexpr int kStageMinPoints = 256;
+
+// The cluster's direction range (DirRange) from this thread's own rows: each
+// warp's part into cs.red_d; the caller's next barrier is followed by
+// direction_range_finish.
+template <int DIM>
+__device__ __forceinline__ void direction_range(const TileRowsOf<DIM> rows, int N, ClusterShared& cs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int hv[4], c = 0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int i = 4 * tid + k;
-    int h = i < n ? (int)S.list[i] : (int)kDropped;
-    if (h != (int)kDropped && !keep(h)) {
-      S.list[i] = kDropped;
-      h = (int)kDropped;
-    }
-    hv[k] = h;
-    c += h != (int)kDropped ? 1 : 0;
+  const float inf = __int_as_float(0x7f800000);
+  float a0 = inf, t0 = inf, t1 = -inf, z = 0.0f;
+  for (int j = tid; j < N; j += kThreads) {
+    const float4 p = rows.at(j);
+    const float t = p.y * rcp_approx(p.x);
+    a0 = fminf(a0, p.x);
+    t0 = fminf(t0, t);
+    t1 = fmaxf(t1, t);
+    if (DIM == 3) z = fmaxf(z, fabsf(p.z));
   }
-  int incl = c;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += t;
+  const int r0 = __reduce_min_sync(0xffffffffu, float_order(a0)), r1 = __reduce_min_sync(0xffffffffu, float_order(t0)),
+            r2 = __reduce_max_sync(0xffffffffu, float_order(t1)),
+            r3 = DIM == 3 ? __reduce_max_sync(0xffffffffu, float_order(z)) : 0;
+  if (lane == 0) {
+    cs.red_d[0][warp] = r0;
+    cs.red_d[1][warp] = r1;
+    cs.red_d[2][warp] = r2;
+    cs.red_d[3][warp] = r3;
   }
-  if (lane == 31) red[warp] = incl;
-  __syncthreads();
-  int pos = incl - c, tot = 0;
-#pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
-    const int v = red[w];
-    tot += v;
-    pos += w < warp ? v : 0;
-  }
-  if (((tot + 127) >> 7) == ((n + 127) >> 7)) return n;  // as many groups: keep the marks
-  // every entry was read before the barrier above: compact in place
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (hv[k] != (int)kDropped) S.list[pos++] = (uint16_t)hv[k];
-  __syncthreads();
-  return tot;
 }
 
-// Staged scoring pass: the first stage covers kStageQuads quads (4 points
-// each), every later one half as many again as the one before; clusters
-// of fewer than kStageMinPoints points are scored in one pass (measured:
-// below that the stages cost more than pruning saves).
-constexpr int kStageQuads = 32;
-constexpr int kStageMinPoints = 512;
+template <int DIM>
+__device__ __forceinline__ void direction_range_finish(bool line, ClusterShared& cs) {
+  if (threadIdx.x != 0) return;
+  int r[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    r[i] = cs.red_d[i][0];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) r[i] = i < 2 ? min(r[i], cs.red_d[i][w]) : max(r[i], cs.red_d[i][w]);
+  }
+  const float a0 = order_float(r[0]), t0 = order_float(r[1]), t1 = order_float(r[2]);
+  const float inv = __fdividef(kTanBins - 0.01f, t1 - t0);
+  cs.dir.t0 = t0;
+  cs.dir.tinv = t1 > t0 && inv < 1e30f ? inv : 0.0f;  // else one bin holds them all
+  cs.dir.tabs = fmaxf(fabsf(t0), fabsf(t1));
+  cs.dir.a0inv = rcp_approx(a0) * kRcpUp;
+  cs.dir.zmax = DIM == 3 ? order_float(r[3]) : 0.0f;
+  cs.dir.tan_ok = !line && a0 > 1e-3f && a0 < 2.0f;
+}
+
+// Scores the chunk's normal trials in stages.  After the first stage the
+// trial with the highest partial count becomes the lead (a later chunk
+// starts from the lead it finds); one pass over the points counts the lead
+// and takes the histograms of its residuals over the points still to be
+// scored.  A trial whose partial count plus the points still to come that it
+// can hold (lead_bound, its counts per stage) cannot beat the lead's key
+// leaves the list, U = -1.  That sum is no less than the trial's exact
+// count, and the lead is ranked by the points it certainly holds, so a trial
+// dropped this way cannot win: the winner is the one that scoring every
+// trial over every point gives, found by the best-first counts among the
+// trials that stayed.  Returns the (trial, point) pairs scored by this warp.
+template <int DIM, bool EXT>
+__device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, const TileRowsOf<DIM> rows,
+                                                          const Smem& S, ClusterShared& cs, int hc0, int nh, int N,
+                                                          unsigned long long* n_cand) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool line = EXT && DIM == 2 && a.line_model;
+  const int nq = (N + 3) >> 2;
+  unsigned long long scored = 0;
+  unsigned top = 0;
+  // pieces of (trial group, quad) units of quads [qa, qb), split evenly over the warps
+  auto score = [&](auto listed, int A, int qa, int qb) {
+    constexpr int G = 32 * kStagedHpl<decltype(listed)::value>;
+    const int span = qb - qa, total = ((A + G - 1) / G) * span;
+    const int per = (total + kWarps - 1) / kWarps;
+    for (int u = warp * per, e = min(total, u + per); u < e;) {
+      const int g = u / span, a0 = qa + u % span, a1 = min(qb, a0 + (e - u));
+      scored += score_segment<DIM, decltype(listed)::value>(rows, N, S, A, g, a0, a1, &top);
+      u += a1 - a0;
+    }
+  };
+  if (tid < 2 * (kTanBins + 1)) cs.lead_in[tid] = 0u;
+  if (tid < 2 * kExcessBins) cs.lead_out[tid] = 0u;
+  unsigned long long lim = cs.best;  // the key to beat
+  int q0 = 0, lead = -1;
+  float4 lw = cs.win;
+  if (lim == 0ull || !(lw.w < 1e30f)) {  // no lead with an FP32 record yet
+    score(std::false_type{}, nh, 0, kStage0Quads);
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) cs.red_i[warp] = (int)top;
+    __syncthreads();
+    top = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) top = max(top, (unsigned)cs.red_i[w]);
+    if (top == 0u) return scored;  // no normal trial
+    q0 = kStage0Quads;
+    lead = 0xFFFF - (int)(top & 0xFFFFu);
+    lw = S.hyp[lead];
+  } else {
+    __syncthreads();
+  }
+  const int e1 = q0 + kStage1Quads, e2 = e1 + 2 * kStage1Quads, e3 = e2 + 4 * kStage1Quads;
+  const DirRange dir = cs.dir;
+  const float ltlo = record_tlo(lw, a.tau32, line);
+  {
+    // the lead's count and the histograms
+    unsigned cnt = 0;  // certain and band points in 16-bit halves
+    for (int j = tid; j < N; j += kThreads) {
+      const float4 p = rows.at(j);
+      const float r = fabsf(resid_f32<DIM>(p, lw.x, lw.y, lw.z));
+      if (r <= ltlo) cnt += 1u;
+      else if (!(r > lw.w)) cnt += 1u << 16;
+      const int q = j >> 2;
+      if (q >= q0) {
+        const unsigned one = (q < e1 || (q >= e2 && q < e3)) ? 1u : 1u << 16;
+        if (r <= lw.w)
+          atomicAdd(&cs.lead_in[(q < e2 ? 0 : kTanBins + 1) + tan_bin(dir, p.y * rcp_approx(p.x))], one);
+        else if (r > lw.w)  // NaN: held by no trial
+          atomicAdd(&cs.lead_out[(q < e2 ? 0 : kExcessBins) + excess_bin(r - lw.w)], one);
+      }
+    }
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) cs.red_i[warp] = (int)cnt;
+    __syncthreads();
+    if (warp < 2) {
+      unsigned* h = warp == 0 ? cs.lead_in : cs.lead_out;
+      const int stride = warp == 0 ? kTanBins + 1 : kExcessBins;
+      const int b = warp == 0 ? lane : 2 * lane;
+      uint2 c0 = make_uint2(h[b], h[stride + b]), c1 = make_uint2(0u, 0u);
+      if (warp == 1) c1 = make_uint2(h[b + 1], h[stride + b + 1]);
+      uint2 incl = make_uint2(c0.x + c1.x, c0.y + c1.y);
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const unsigned tx = __shfl_up_sync(0xffffffffu, incl.x, d), ty = __shfl_up_sync(0xffffffffu, incl.y, d);
+        if (lane >= d) {
+          incl.x += tx;
+          incl.y += ty;
+        }
+      }
+      auto put = [&](int bin, unsigned x, unsigned y) {
+        y += y >> 16;              // stages 2 and 3, 3
+        x += (y & 0xFFFFu) << 16;  // 1 on
+        x += x >> 16;              // 0 on
+        h[bin] = x;
+        h[stride + bin] = y;
+      };
+      if (warp == 0) {
+        put(lane, incl.x - c0.x, incl.y - c0.y);
+        if (lane == 31) put(kTanBins, incl.x, incl.y);
+      } else {
+        put(b, incl.x - c1.x, incl.y - c1.y);
+        put(b + 1, incl.x, incl.y);
+      }
+    } else if (warp == 2) {
+      const unsigned v = __reduce_add_sync(0xffffffffu, lane < kWarps ? (unsigned)cs.red_i[lane] : 0u);
+      if (lane == 0) cs.lead_cnt = v;
+    }
+    __syncthreads();
+  }
+  if (lead >= 0) {
+    const int certain = (int)(cs.lead_cnt & 0xFFFFu), near = (int)(cs.lead_cnt >> 16);
+    const unsigned long long key = best_key(certain, hc0 + lead);
+    if (tid == 0) {
+      if (near == 0) {  // counted exactly: it leaves the pool
+        S.U[lead] = -1;
+        if (key > lim) {
+          cs.best = key;
+          cs.win = lw;
+          cs.win_has_v64 = 0;
+        }
+        ++*n_cand;
+      } else {
+        S.U[lead] = certain + near;
+      }
+    }
+    lim = max(lim, key);
+  }
+  const float lead_band = record_band(lw, a.tau32.hi, line);
+  // the pruning test before stage s: the points from it on that trial h can hold
+  auto keep = [&](int h, HoldRange r, int s) {
+    const int sh = (s & 1) << 4;
+    const unsigned* in = cs.lead_in + (s >> 1) * (kTanBins + 1);
+    const unsigned* out = cs.lead_out + (s >> 1) * kExcessBins;
+    const int n = (int)(out[r.out()] >> sh & 0xFFFFu) + (int)(in[r.hi()] >> sh & 0xFFFFu) -
+                  (int)(in[r.lo()] >> sh & 0xFFFFu);
+    const bool k = best_key(S.U[h] + n, hc0 + h) > lim;
+    if (!k) S.U[h] = -1;
+    return k;
+  };
+  int A = prune_list<false>(
+      S, nh,
+      [&](int h) {
+        if (h == lead) return false;  // its count is already known
+        const HoldRange r = hold_range<DIM>(dir, lw, lead_band, a.tau32.hi, line, S.hyp[h]);
+        S.tlo[h] = __uint_as_float(r.v);
+        return keep(h, r, 0);
+      },
+      cs.red_i);
+  for (int s = 1; A > 0 && q0 < nq; ++s) {
+    const int q1 = s == 1 ? e1 : (s == 2 ? e2 : (s == 3 ? e3 : nq));
+    const bool last = s == 4 || q1 + (q1 - q0) / 2 >= nq;  // no short last stage
+    score(std::true_type{}, A, q0, last ? nq : q1);
+    if (last) break;
+    __syncthreads();
+    q0 = q1;
+    A = prune_list<true>(
+        S, A, [&](int h) { return keep(h, HoldRange{__float_as_uint(S.tlo[h])}, s); }, cs.red_i);
+  }
+  return scored;
+}
 
 // a2 + a3 for trials hc0 .. hc0 + nh - 1 of cluster ci under the cosine
 // model: draw, FP32 solve (refined when ill-conditioned), bound, records
@@ -919,7 +1165,6 @@ __device__ __forceinline__ void cosine_trial_chunk(const FrameDesc& a, const RV 
     if (hy.kind == kHypExactOnly) ++n_fp64;
     n_ref += hy.refined;
     S.hyp[hl] = make_float4(hy.nx, hy.ny, hy.nz, hy.kind == kHypRejected ? __int_as_float(0x7fc00000) : hy.thi);
-    S.tlo[hl] = hy.tlo;
     S.kind[hl] = (int8_t)hy.kind;
     if constexpr (DIM == 2) {
       // the queue lives in U until the second pass has read it
@@ -950,8 +1195,7 @@ __device__ __forceinline__ void cosine_trial_chunk(const FrameDesc& a, const RV 
       }
       n_ref += hy.refined;
       S.hyp[hl] = make_float4(hy.nx, hy.ny, hy.nz, hy.thi);
-      S.tlo[hl] = hy.tlo;
-      S.kind[hl] = (int8_t)hy.kind;
+        S.kind[hl] = (int8_t)hy.kind;
     }
     __syncthreads();
     for (int hl = tid; hl < nh; hl += kThreads) {
@@ -1036,14 +1280,17 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
       rows.put(N + tid, make_float4(0.0f, 0.0f, nan, nan));
     }
   }
-  wm = block_max_float(wm, cs.red_f);  // includes a __syncthreads after the row writes
   if (tid == 0) {
     cs.best = 0ull;
-    cs.wmax = wm;
     cs.nref = 0;
   }
-  __syncthreads();
-  const float wmax = cs.wmax;
+  if constexpr (SMEM_ROWS) {
+    if (N >= kStageMinPoints) direction_range<DIM>(rows, N, cs);
+  }
+  const float wmax = block_max_float(wm, cs.red_f);  // its barrier also orders the row writes
+  if constexpr (SMEM_ROWS) {
+    if (N >= kStageMinPoints) direction_range_finish<DIM>(EXT && DIM == 2 && a.line_model, cs);
+  }
   unsigned long long n_fp64 = 0, n_cand = 0, n_ref = 0, n_scored = 0;
   stage_done(0);
 
@@ -1072,8 +1319,7 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
           }
           if (hy.kind == kHypExactOnly) ++n_fp64;
           S.hyp[hl] = make_float4(hy.nx, hy.ny, hy.nz, hy.kind == kHypRejected ? __int_as_float(0x7fc00000) : hy.thi);
-          S.tlo[hl] = hy.tlo;
-          S.kind[hl] = (int8_t)hy.kind;
+                S.kind[hl] = (int8_t)hy.kind;
           S.U[hl] = hy.kind == kHypRejected ? -1 : (hy.kind == kHypExactOnly ? N : 0);
         }
       } else {
@@ -1090,7 +1336,7 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
     // becomes the lead if its key beats it
     auto count_trial = [&](int c) {
       const float4 hy = S.hyp[c];
-      const float htlo = S.tlo[c];
+      const float htlo = record_tlo(hy, a.tau32, EXT && DIM == 2 && a.line_model);
       int B = 0;
       const int C = exact_count_block<DIM, RV, EXT>(a, rows, R, ci, hc0 + c, N, hy, htlo, cs, &B);
       ++n_cand;
@@ -1100,7 +1346,6 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
         if (k > cs.best) {
           cs.best = k;
           cs.win = hy;
-          cs.win_tlo = htlo;
           cs.win_has_v64 = B > 0;
           cs.win_v64[0] = cs.cv64[0];
           cs.win_v64[1] = cs.cv64[1];
@@ -1117,57 +1362,7 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
       phase_a_dispatch<DIM>(pw, hpl, rows, N, S, nh);
       if (tid == 0) n_scored += (unsigned long long)nh * (unsigned long long)N;
     } else if constexpr (SMEM_ROWS) {
-      // Staged, with exact pruning: the trials still in the list are scored
-      // in stages (kStageQuads quads, then each stage half as long again);
-      // after the first stage the trial with the highest partial count is
-      // counted exactly (it leads from then on), and after every stage a
-      // trial whose partial count plus the points still to come cannot beat
-      // the lead's key leaves the list (U = -1; marked kDropped, or
-      // compacted away).  Each remaining point adds at most one to a count and
-      // C_h <= U_h, so a trial dropped this way cannot win: the winner is
-      // the one scoring every trial over every point gives, found by the
-      // best-first counts below among the trials that stayed.
-      const int nq = (N + 3) >> 2;
-      int A = compact_list(S, nh, false, [&](int h) { return S.kind[h] == kHypNormal; }, cs.red_i);
-      bool led = false;
-      unsigned long long scored = 0;
-      int sq = kStageQuads;
-      for (int q0 = 0; q0 < nq && A > 0;) {
-        int q1 = min(nq, q0 + sq);
-        if (nq - q1 < sq / 2) q1 = nq;  // no short last stage
-        sq = (sq * 3) >> 1;
-        // (trial group, quad) units split evenly over the warps
-        const int span = q1 - q0, total = ((A + 127) >> 7) * span;
-        const int per = (total + kWarps - 1) / kWarps;
-        for (int u = (tid >> 5) * per, e = min(total, u + per); u < e;) {
-          const int g = u / span, qa = q0 + u % span, qb = min(q0 + span, qa + (e - u));
-          scored += (unsigned long long)score_segment<DIM>(rows, N, S, A, g, qa, qb);
-          u += qb - qa;
-        }
-        __syncthreads();
-        q0 = q1;
-        if (q0 >= nq) break;
-        const int rem = N - 4 * q0;
-        if (!led) {
-          led = true;
-          unsigned long long km = 0;
-          for (int i = tid; i < A; i += kThreads) {
-            const int h = S.list[i];
-            if (h != (int)kDropped) km = max(km, best_key(S.U[h], hc0 + h));
-          }
-          km = block_max_u64(km, cs.red_u);
-          const int c = (int)(0xFFFFFFFFu - (uint32_t)(km & 0xFFFFFFFFull)) - hc0;
-          if (km != 0ull && best_key(S.U[c] + rem, hc0 + c) > cs.best) count_trial(c);
-        }
-        const unsigned long long lead = cs.best;
-        auto alive = [&](int h) {
-          const int u = S.U[h];
-          const bool keep = u >= 0 && best_key(u + rem, hc0 + h) > lead;
-          if (!keep) S.U[h] = -1;
-          return keep;
-        };
-        A = A <= 4 * kThreads ? prune_list(S, A, alive, cs.red_i) : compact_list(S, A, true, alive, cs.red_i);
-      }
+      const unsigned long long scored = staged_pass<DIM, EXT>(a, rows, S, cs, hc0, nh, N, &n_cand);
       if ((tid & 31) == 0) n_scored += scored;
     }
     __syncthreads();
@@ -1182,12 +1377,15 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
     // give.  Trials of earlier chunks have lower indices; the lead's key
     // already ranks them.  A counted trial leaves the pool (U = -1).
     for (;;) {
-      unsigned long long km = 0;
+      int um = -1, hm = 0x7fffffff;
       for (int hl = tid; hl < nh; hl += kThreads) {
         const int u = S.U[hl];
-        if (u >= 0) km = max(km, best_key(u, hc0 + hl));
+        if (u > um) {
+          um = u;
+          hm = hc0 + hl;
+        }
       }
-      km = block_max_u64(km, cs.red_u);
+      const unsigned long long km = block_best(um, hm, cs.red_u);
       if (km <= cs.best) break;  // also km == 0: no trial left
       count_trial((int)(0xFFFFFFFFu - (uint32_t)(km & 0xFFFFFFFFull)) - hc0);
     }
@@ -1230,7 +1428,7 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
   // whose FP64 velocity was computed when it was counted) and the normal
   // equations over its inliers.
   const float4 win = cs.win;
-  const float wtlo = cs.win_tlo;
+  const float wtlo = record_tlo(win, a.tau32, EXT && DIM == 2 && a.line_model);
   const double v64[3] = {cs.win_v64[0], cs.win_v64[1], cs.win_v64[2]};
   constexpr int NS = DIM == 2 ? 5 : 9;
   int n_in = mask_and_sums<DIM, RV, EXT>(a, rows, R, o, N, win, wtlo, v64, S, cs, false, nullptr);

@@ -23,7 +23,7 @@ constexpr int kWarps = kThreads / 32;
 struct Smem {
   float* rows;        // [roundup32(nmax_smem) * 4] floats of row tiles (TileRows)
   float4* hyp;        // [hchunk] (-X, -Y, -Z, thi)
-  float* tlo;         // [hchunk]
+  float* tlo;         // [hchunk] staged pass: what each trial can hold (HoldRange, as bits)
   int* U;             // [hchunk] upper bounds of the exact counts (-1 = rejected)
   int8_t* kind;       // [hchunk]
   uint16_t* list;     // [hchunk] trials still scored by the staged pass
@@ -215,37 +215,53 @@ __device__ __forceinline__ void phase_a_tiles(const TileRowsOf<DIM> rows, int N,
   }
 }
 
-// A list entry of a trial dropped in place (the list is compacted only when
-// that saves a group of 128).
-constexpr uint16_t kDropped = 0xFFFF;
+// Trial at position i of the staged pass's list, -1 past its end.  LISTED =
+// false: there is no list yet, position i is trial i, and trials without a
+// normal record (rejected, or counted only in FP64) are passed over.
+template <bool LISTED>
 __device__ __forceinline__ int list_trial(const Smem& S, int A, int i) {
-  const int e = i < A ? (int)S.list[i] : (int)kDropped;
-  return e == (int)kDropped ? -1 : e;
+  if (i >= A) return -1;
+  return LISTED ? (int)S.list[i] : (S.kind[i] == kHypNormal ? i : -1);
 }
 
-// One piece of the staged scoring pass: the 128 trials of group g of the
-// list S.list[0 .. A) (four per lane, lane-major) over quads [qa, qb),
-// their counts added to S.U (several warps may share a group, each over
-// its own quads).  Returns the (trial, point) pairs this warp scored.
-template <int DIM>
-__device__ __forceinline__ long long score_segment(const TileRowsOf<DIM> rows, int N, const Smem& S, int A, int g,
-                                                   int qa, int qb) {
+// Trials per lane of the staged pass: four while every trial is scored, two
+// for the lists that pruning leaves -- groups of 64 trials instead of 128
+// waste fewer lanes on a list's end, which outweighs the point rows being
+// loaded for half as many trials (dense2d 0.2275 -> 0.2233 ms, stress2d 0.848
+// -> 0.802 ms; one trial per lane 0.2326 / 0.813 ms).
+template <bool LISTED>
+constexpr int kStagedHpl = LISTED ? 2 : 4;
+
+// One piece of the staged scoring pass: the 32 kStagedHpl trials of group g
+// of the list (lane-major) over quads [qa, qb), their counts added to S.U
+// (several warps may share a group, each over its own quads).  *top
+// (unlisted trials) collects the lane's highest count in its upper half and
+// the trial, as 0xFFFF - h, in its lower one.  Returns the (trial, point)
+// pairs this warp scored.
+template <int DIM, bool LISTED>
+__device__ __forceinline__ unsigned score_segment(const TileRowsOf<DIM> rows, int N, const Smem& S, int A, int g,
+                                                  int qa, int qb, unsigned* top) {
   const int lane = threadIdx.x & 31;
-  LaneTrials<4> T;
-  int hs[4];
+  constexpr int HPL = kStagedHpl<LISTED>;
+  LaneTrials<HPL> T;
+  int hs[HPL];
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    hs[m] = list_trial(S, A, g * 128 + lane * 4 + m);
+  for (int m = 0; m < HPL; ++m) {
+    hs[m] = list_trial<LISTED>(S, A, g * 32 * HPL + lane * HPL + m);
     T.load(m, hs[m] >= 0 ? S.hyp[hs[m]] : make_float4(0.f, 0.f, 0.f, __int_as_float(0x7fc00000)));
   }
-  score_quads<DIM, 4>(rows, qa, qb, 1, T);
+  score_quads<DIM, HPL>(rows, qa, qb, 1, T);
   int trials = 0;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    if (hs[m] >= 0) atomicAdd(&S.U[hs[m]], sign_count(T.acc[m]));
-    trials += __popc(__ballot_sync(0xffffffffu, hs[m] >= 0));
+  for (int m = 0; m < HPL; ++m) {
+    if (hs[m] >= 0) {
+      const int c = sign_count(T.acc[m]);
+      atomicAdd(&S.U[hs[m]], c);
+      if (!LISTED) *top = max(*top, ((unsigned)c << 16) | (unsigned)(0xFFFF - hs[m]));
+      ++trials;
+    }
   }
-  return (long long)trials * (min(4 * qb, N) - 4 * qa);
+  return (unsigned)__reduce_add_sync(0xffffffffu, trials) * (unsigned)(min(4 * qb, N) - 4 * qa);
 }
 
 }  // namespace rvh
