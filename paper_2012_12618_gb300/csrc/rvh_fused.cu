@@ -74,76 +74,20 @@ __device__ __forceinline__ float block_max_float(float v, int* red) {
   return __int_as_float(r);
 }
 
-// ---- a4: upper-bound counts U_h = #{|r32| <= thi_h} (the hot loop) -----------------
-// Lane l handles trial sub-group l / PW and points l % PW, l % PW + PW, ...;
-// each lane keeps HPL trials in registers.  PW = 32 is warp-per-trial-group
-// with lanes over points; PW = 1 is lanes over trials with broadcast rows.
-template <int DIM, int PW, int HPL>
-__device__ __forceinline__ void phase_a(const float4* __restrict__ rows, int N, const Smem& S, int nh) {  // global rows
-  constexpr int NHL = 32 / PW;
-  constexpr int G = NHL * HPL;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int hl = lane / PW, pl = lane % PW;
-  const int ngroups = (nh + G - 1) / G;
-  for (int g = warp; g < ngroups; g += kWarps) {
-    const int base = g * G + hl * HPL;
-    float nx[HPL], ny[HPL], nz[HPL], th[HPL], cnt[HPL];
-#pragma unroll
-    for (int m = 0; m < HPL; ++m) {
-      const int h = base + m;
-      float4 v = (h < nh) ? S.hyp[h] : make_float4(0.f, 0.f, 0.f, __int_as_float(0x7fc00000));
-      nx[m] = v.x;
-      ny[m] = v.y;
-      nz[m] = v.z;
-      th[m] = v.w;
-      cnt[m] = 0.0f;
-    }
-    for (int j = pl; j < N; j += PW) {
-      const float4 p = rows[j];
-#pragma unroll
-      for (int m = 0; m < HPL; ++m) {
-        const float r = resid_f32<DIM>(p, nx[m], ny[m], nz[m]);
-        cnt[m] += (fabsf(r) <= th[m]) ? 1.0f : 0.0f;
-      }
-    }
-#pragma unroll
-    for (int m = 0; m < HPL; ++m) {
-#pragma unroll
-      for (int o = PW / 2; o > 0; o >>= 1) cnt[m] += __shfl_xor_sync(0xffffffffu, cnt[m], o);
-    }
-    if (pl == 0) {
-#pragma unroll
-      for (int m = 0; m < HPL; ++m) {
-        const int h = base + m;
-        if (h < nh && S.kind[h] == kHypNormal) S.U[h] = (int)cnt[m];
-      }
-    }
-  }
-}
-
-// The tiled pass keeps four trials per lane whatever hpl asks: eight packed
-// trials (pairs of registers per coordinate) do not fit in the 64 registers a
-// thread has at four CTAs per SM.
-template <int DIM>
-__device__ void phase_a_dispatch(int pw, int hpl, const TileRowsOf<DIM> rows, int N, const Smem& S, int nh) {
-  (void)hpl;
+// ---- a4: upper-bound counts U_h = #{|r32| <= thi_h} of every trial (the hot loop) --
+// Lane l handles trial sub-group l / pw and point quads l % pw, l % pw + pw,
+// ...: pw = 32 is warp-per-trial-group with lanes over points, pw = 1 lanes
+// over trials with broadcast rows.  Four trials per lane whatever
+// hyps_per_lane asks: eight packed trials (pairs of registers per
+// coordinate) do not fit in the 64 registers a thread has at four CTAs per SM.
+template <int DIM, typename RV>
+__device__ void phase_a_dispatch(int pw, const RV rows, int N, const Smem& S, int nh) {
   if (pw == 1) {
     phase_a_tiles<DIM, 1, 4>(rows, N, S, nh);
   } else if (pw == 8) {
     phase_a_tiles<DIM, 8, 4>(rows, N, S, nh);
   } else {
     phase_a_tiles<DIM, 32, 4>(rows, N, S, nh);
-  }
-}
-
-template <int DIM>
-__device__ void phase_a_dispatch(int pw, int hpl, const AosRows rows, int N, const Smem& S, int nh) {
-  if (pw == 1) {
-    if (hpl == 8) phase_a<DIM, 1, 8>(rows.p, N, S, nh); else phase_a<DIM, 1, 4>(rows.p, N, S, nh);
-  } else if (pw == 8) {
-    if (hpl == 8) phase_a<DIM, 8, 8>(rows.p, N, S, nh); else phase_a<DIM, 8, 4>(rows.p, N, S, nh);
-  } else {
-    if (hpl == 8) phase_a<DIM, 32, 8>(rows.p, N, S, nh); else phase_a<DIM, 32, 4>(rows.p, N, S, nh);
   }
 }
 
@@ -911,12 +855,13 @@ __device__ __forceinline__ int prune_list(const Smem& S, int n, Keep keep, int* 
 // early stage evaluates fewer pairs (29%) but took 0.305 ms.
 constexpr int kStage0Quads = 32, kStage1Quads = 32;
 constexpr int kStageMinPoints = 256;
+constexpr int kStageMaxPoints = 32767;  // points are counted in 16-bit halves
 
 // The cluster's direction range (DirRange) from this thread's own rows: each
 // warp's part into cs.red_d; the caller's next barrier is followed by
 // direction_range_finish.
-template <int DIM>
-__device__ __forceinline__ void direction_range(const TileRowsOf<DIM> rows, int N, ClusterShared& cs) {
+template <int DIM, typename RV>
+__device__ __forceinline__ void direction_range(const RV rows, int N, ClusterShared& cs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float inf = __int_as_float(0x7f800000);
   float a0 = inf, t0 = inf, t1 = -inf, z = 0.0f;
@@ -970,9 +915,9 @@ __device__ __forceinline__ void direction_range_finish(bool line, ClusterShared&
 // dropped this way cannot win: the winner is the one that scoring every
 // trial over every point gives, found by the best-first counts among the
 // trials that stayed.  Returns the (trial, point) pairs scored by this warp.
-template <int DIM, bool EXT>
-__device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, const TileRowsOf<DIM> rows,
-                                                          const Smem& S, ClusterShared& cs, int hc0, int nh, int N,
+template <int DIM, bool EXT, typename RV>
+__device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, const RV rows, const Smem& S,
+                                                          ClusterShared& cs, int hc0, int nh, int N,
                                                           unsigned long long* n_cand) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool line = EXT && DIM == 2 && a.line_model;
@@ -1210,8 +1155,8 @@ __device__ __forceinline__ void cosine_trial_chunk(const FrameDesc& a, const RV 
 
 template <int DIM, bool SMEM_ROWS, bool EXT>
 __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared& cs, int ci, int hchunk,
-                                int pw, int hpl, int prune, int frame, FinishRec* fq, int* fq_n,
-                                double4_32a* cta_pre) {
+                                int pw, int prune, int frame, FinishRec* fq, int* fq_n,
+                                double4_32a* cta_pre, int row_cap) {
   const int tid = threadIdx.x;
   const int64_t o = a.offsets[ci];
   const int64_t e = a.offsets[ci + 1];
@@ -1225,12 +1170,17 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
     if (tid == 0) write_invalid<DIM>(a, ci, RVH_STATUS_TOO_FEW_POINTS);
     return;
   }
-  using RV = typename std::conditional<SMEM_ROWS, TileRowsOf<DIM>, AosRows>::type;
+  using RV = typename std::conditional<SMEM_ROWS, TileRowsOf<DIM>, HybridRowsOf<DIM>>::type;
   RV rows;
   if constexpr (SMEM_ROWS) {
     rows.f = S.rows;
   } else {
-    rows.p = a.rows_g + o;
+    // the tail's tiles start at the cluster's own float4 [N] region, whose
+    // cap unused entries leave room for rounding its end up
+    constexpr int NC = DIM == 2 ? 3 : 4;
+    rows.s.f = S.rows;
+    rows.cap = row_cap;
+    rows.g.f = reinterpret_cast<float*>(a.rows_g + o) - (size_t)row_cap * NC;
   }
   // FP64 rows: the CTA's own slot when the cluster fits it (the slot is
   // reused cluster after cluster and stays in L2), else the frame's
@@ -1273,24 +1223,19 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
   } else {
     cosine_rows();
   }
-  if constexpr (SMEM_ROWS) {
-    // pad the last quad of the scoring pass: NaN Dopplers never count
-    if (tid < ((N + 3) & ~3) - N) {
-      const float nan = __int_as_float(0x7fc00000);
-      rows.put(N + tid, make_float4(0.0f, 0.0f, nan, nan));
-    }
+  // pad the last quad of the scoring pass: NaN Dopplers never count
+  if (tid < ((N + 3) & ~3) - N) {
+    const float nan = __int_as_float(0x7fc00000);
+    rows.put(N + tid, make_float4(0.0f, 0.0f, nan, nan));
   }
   if (tid == 0) {
     cs.best = 0ull;
     cs.nref = 0;
   }
-  if constexpr (SMEM_ROWS) {
-    if (N >= kStageMinPoints) direction_range<DIM>(rows, N, cs);
-  }
+  const bool may_stage = prune && pw == 1 && N >= kStageMinPoints && N <= kStageMaxPoints;
+  if (may_stage) direction_range<DIM>(rows, N, cs);
   const float wmax = block_max_float(wm, cs.red_f);  // its barrier also orders the row writes
-  if constexpr (SMEM_ROWS) {
-    if (N >= kStageMinPoints) direction_range_finish<DIM>(EXT && DIM == 2 && a.line_model, cs);
-  }
+  if (may_stage) direction_range_finish<DIM>(EXT && DIM == 2 && a.line_model, cs);
   unsigned long long n_fp64 = 0, n_cand = 0, n_ref = 0, n_scored = 0;
   stage_done(0);
 
@@ -1356,14 +1301,12 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
     };
 
     // a4: scoring pass (the hot loop)
-    bool staged = false;
-    if constexpr (SMEM_ROWS) staged = prune && pw == 1 && N >= kStageMinPoints;
-    if (!staged) {
-      phase_a_dispatch<DIM>(pw, hpl, rows, N, S, nh);
-      if (tid == 0) n_scored += (unsigned long long)nh * (unsigned long long)N;
-    } else if constexpr (SMEM_ROWS) {
+    if (may_stage) {
       const unsigned long long scored = staged_pass<DIM, EXT>(a, rows, S, cs, hc0, nh, N, &n_cand);
       if ((tid & 31) == 0) n_scored += scored;
+    } else {
+      phase_a_dispatch<DIM>(pw, rows, N, S, nh);
+      if (tid == 0) n_scored += (unsigned long long)nh * (unsigned long long)N;
     }
     __syncthreads();
     stage_done(2);
@@ -1527,10 +1470,11 @@ __global__ void __launch_bounds__(kThreads, RVH_MIN_BLOCKS) fused_kernel(const _
     const int64_t o = F.offsets[ci], e = F.offsets[ci + 1];
     double4_32a* cta_pre =
         a.cta_rows64 ? a.cta_rows64 + (size_t)blockIdx.x * cta_slot_stride(DIM, a.nmax_smem) : nullptr;
-    if (e - o <= (int64_t)smem_row_capacity(DIM, a.nmax_smem) || e < o) {
-      process_cluster<DIM, true, EXT>(F, S, cs, ci, a.hchunk, a.pw, a.hpl, a.prune, fc.x, fq, &fq_n, cta_pre);
+    const int cap = smem_row_capacity(DIM, a.nmax_smem);
+    if (e - o <= (int64_t)cap || e < o) {
+      process_cluster<DIM, true, EXT>(F, S, cs, ci, a.hchunk, a.pw, a.prune, fc.x, fq, &fq_n, cta_pre, cap);
     } else {
-      process_cluster<DIM, false, EXT>(F, S, cs, ci, a.hchunk, a.pw, a.hpl, a.prune, fc.x, fq, &fq_n, cta_pre);
+      process_cluster<DIM, false, EXT>(F, S, cs, ci, a.hchunk, a.pw, a.prune, fc.x, fq, &fq_n, cta_pre, cap & ~31);
     }
     __syncthreads();
     if (fq_n == kFinishBatch) flush();

@@ -8,6 +8,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 #include "rvh_device.cuh"
@@ -35,8 +36,7 @@ struct Smem {
 // warp reading consecutive points touches 32 banks per component, and four
 // consecutive points of one component are one aligned float4, which the
 // scoring pass consumes as two packed pairs.  NC = 3 (2D) or 4 (3D)
-// components; at() of a 2D row leaves .w zero.  Clusters larger than the
-// shared memory area keep plain float4 rows in global scratch.
+// components; at() of a 2D row leaves .w zero.
 template <int NC>
 struct TileRows {
   float* f;
@@ -59,11 +59,27 @@ struct TileRows {
 template <int DIM>
 using TileRowsOf = TileRows<DIM == 2 ? 3 : 4>;
 
-struct AosRows {
-  float4* p;
-  __device__ __forceinline__ float4 at(int j) const { return p[j]; }
-  __device__ __forceinline__ void put(int j, float4 v) const { p[j] = v; }
+// Rows of a cluster larger than the shared-memory area: the first cap points
+// (a multiple of 32) in shared memory, the others in global scratch, in the
+// same tiles (g is offset so that both use the same index).  The staged pass
+// scores most trials over the first points only, so the tail is read by the
+// few that stay.  Such a cluster used to keep all its rows in global memory,
+// read point by point and unstaged, and set the length of a small 3D frame:
+// 1025 clusters of 8..2048 points at 2048 trials 0.625 -> 0.353 ms.
+template <int NC>
+struct HybridRows {
+  TileRows<NC> s;
+  TileRows<NC> g;
+  int cap;
+  __device__ __forceinline__ float4 at(int j) const { return j < cap ? s.at(j) : g.at(j); }
+  __device__ __forceinline__ void put(int j, float4 v) const {
+    if (j < cap) s.put(j, v);
+    else g.put(j, v);
+  }
+  __device__ __forceinline__ float4 quad(int q, int k) const { return 4 * q < cap ? s.quad(q, k) : g.quad(q, k); }
 };
+template <int DIM>
+using HybridRowsOf = HybridRows<DIM == 2 ? 3 : 4>;
 
 // Packed FP32 pairs (fma.rn.f32x2 rounds each half like the scalar
 // instruction, so results are those of fmaf per element).
@@ -134,10 +150,9 @@ struct LaneTrials {
 // only loosen the bound).  The count leaves the FP32 pipe: two byte permutes
 // turn the four sign bits into 16-bit masks and one three-input integer add
 // accumulates them (sign_pair / sign_count: the even and the odd points of a
-// lane stay below 2^16 each, since a cluster in shared memory has at most
-// 227 KB / 12 B points).
-template <int DIM, int HPL>
-__device__ __forceinline__ void score_quad(const TileRowsOf<DIM>& rows, int q, LaneTrials<HPL>& T) {
+// lane stay below 2^16 each: kMaxQuads between two sign_counts).
+template <int DIM, int HPL, typename RV>
+__device__ __forceinline__ void score_quad(const RV& rows, int q, LaneTrials<HPL>& T) {
   const float4 c = rows.quad(q, 0), sn = rows.quad(q, 1), w = rows.quad(q, DIM == 2 ? 2 : 3);
   const unsigned long long c01 = pack2(c.x, c.y), c23 = pack2(c.z, c.w);
   const unsigned long long s01 = pack2(sn.x, sn.y), s23 = pack2(sn.z, sn.w);
@@ -166,23 +181,24 @@ __device__ __forceinline__ void score_quad(const TileRowsOf<DIM>& rows, int q, L
 }
 
 // Quads q0, q0 + step, ... below q1, unrolled by the measured factor.
-template <int DIM, int HPL>
-__device__ __forceinline__ void score_quads(const TileRowsOf<DIM>& rows, int q0, int q1, int step,
+template <int DIM, int HPL, typename RV>
+__device__ __forceinline__ void score_quads(const RV& rows, int q0, int q1, int step,
                                             LaneTrials<HPL>& T) {
   constexpr int UN = DIM == 2 ? 8 : 4;  // quads per loop iteration (measured)
   int q = q0;
   for (; q + (UN - 1) * step < q1; q += UN * step) {
 #pragma unroll
-    for (int u = 0; u < UN; ++u) score_quad<DIM, HPL>(rows, q + u * step, T);
+    for (int u = 0; u < UN; ++u) score_quad<DIM>(rows, q + u * step, T);
   }
-  for (; q < q1; q += step) score_quad<DIM, HPL>(rows, q, T);
+  for (; q < q1; q += step) score_quad<DIM>(rows, q, T);
 }
 
 // a4 over tiled rows, every trial of the chunk over every point.  Lane l
 // handles trial sub-group l / PW and point quads l % PW, l % PW + PW, ...;
 // the rows stage pads the last quad with NaN Dopplers, which never count.
-template <int DIM, int PW, int HPL>
-__device__ __forceinline__ void phase_a_tiles(const TileRowsOf<DIM> rows, int N, const Smem& S, int nh) {
+constexpr int kMaxQuads = 1 << 14;  // quads of one lane whose counts fit sign_count's halves, with margin
+template <int DIM, int PW, int HPL, typename RV>
+__device__ __forceinline__ void phase_a_tiles(const RV rows, int N, const Smem& S, int nh) {
   constexpr int NHL = 32 / PW;
   constexpr int G = NHL * HPL;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -197,11 +213,25 @@ __device__ __forceinline__ void phase_a_tiles(const TileRowsOf<DIM> rows, int N,
       const int h = base + m;
       T.load(m, (h < nh) ? S.hyp[h] : make_float4(0.f, 0.f, 0.f, __int_as_float(0x7fc00000)));
     }
-    score_quads<DIM, HPL>(rows, pl, nq, PW, T);
     int cnt[HPL];
+    if constexpr (std::is_same<RV, TileRowsOf<DIM>>::value) {  // at most 227 KB / 12 B points
+      score_quads<DIM>(rows, pl, nq, PW, T);
+#pragma unroll
+      for (int m = 0; m < HPL; ++m) cnt[m] = sign_count(T.acc[m]);
+    } else {
+#pragma unroll
+      for (int m = 0; m < HPL; ++m) cnt[m] = 0;
+      for (int q0 = 0; q0 < nq; q0 += PW * kMaxQuads) {
+        score_quads<DIM>(rows, q0 + pl, min(nq, q0 + PW * kMaxQuads), PW, T);
+#pragma unroll
+        for (int m = 0; m < HPL; ++m) {
+          cnt[m] += sign_count(T.acc[m]);
+          T.acc[m] = 0u;
+        }
+      }
+    }
 #pragma unroll
     for (int m = 0; m < HPL; ++m) {
-      cnt[m] = sign_count(T.acc[m]);
 #pragma unroll
       for (int o = PW / 2; o > 0; o >>= 1) cnt[m] += __shfl_xor_sync(0xffffffffu, cnt[m], o);
     }
@@ -238,8 +268,8 @@ constexpr int kStagedHpl = LISTED ? 2 : 4;
 // (unlisted trials) collects the lane's highest count in its upper half and
 // the trial, as 0xFFFF - h, in its lower one.  Returns the (trial, point)
 // pairs this warp scored.
-template <int DIM, bool LISTED>
-__device__ __forceinline__ unsigned score_segment(const TileRowsOf<DIM> rows, int N, const Smem& S, int A, int g,
+template <int DIM, bool LISTED, typename RV>
+__device__ __forceinline__ unsigned score_segment(const RV rows, int N, const Smem& S, int A, int g,
                                                   int qa, int qb, unsigned* top) {
   const int lane = threadIdx.x & 31;
   constexpr int HPL = kStagedHpl<LISTED>;
@@ -250,7 +280,7 @@ __device__ __forceinline__ unsigned score_segment(const TileRowsOf<DIM> rows, in
     hs[m] = list_trial<LISTED>(S, A, g * 32 * HPL + lane * HPL + m);
     T.load(m, hs[m] >= 0 ? S.hyp[hs[m]] : make_float4(0.f, 0.f, 0.f, __int_as_float(0x7fc00000)));
   }
-  score_quads<DIM, HPL>(rows, qa, qb, 1, T);
+  score_quads<DIM>(rows, qa, qb, 1, T);
   int trials = 0;
 #pragma unroll
   for (int m = 0; m < HPL; ++m) {

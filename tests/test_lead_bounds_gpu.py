@@ -72,3 +72,26 @@ def test_bounds_keep_every_result(ctx, dim, H):
     # ill-conditioned sets of the narrow and two-direction clusters may sit on a rounding tie the oracle flags
     rep = G.compare(g, o, off)
     assert not rep["mismatch"], rep["mismatch"][:10]
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_rows_beyond_shared_memory(ctx, dim):
+    """Clusters around the staged pass's largest size and past the points one
+    count register holds, their rows split between shared and global memory."""
+    from paper_2012_12618_gb300 import rvh
+    w = synth.WORKLOADS["dense2d" if dim == 2 else "dense3d"]
+    f = synth.make_frame(w, sizes=np.array([1536, 1537, 2080, 32767, 32768, 70001, 9]), gen_seed=31)
+    kw = dict(el=f.elevation, H=96, tau=0.1, seed=3)
+    outs = []
+    for pw, prune in ((1, 1), (1, 0), (8, 1), (32, 1)):
+        assert rvh.rvh_set_schedule(ctx.handle, pw, 4) == 0 and rvh.rvh_set_pruning(ctx.handle, prune) == 0
+        try:
+            outs.append(G.run_rvh(ctx, f.azimuth, f.doppler, f.offsets, **kw))
+        finally:
+            rvh.rvh_set_schedule(ctx.handle, 0, 0)
+            rvh.rvh_set_pruning(ctx.handle, 1)
+    for u in outs[1:]:
+        for k in G.OUT_KEYS:
+            assert np.array_equal(outs[0][k], u[k]), k
+    o = G.run_oracle(f.azimuth, f.doppler, f.offsets, **kw)
+    assert not G.compare(outs[0], o, f.offsets)["mismatch"]
