@@ -314,6 +314,7 @@ int prepare_launch(rvh_ctx* ctx, FusedArgs& a, int dim, int* grid, size_t* smem)
   // when every item gets its own resident CTA the order cannot matter: skip
   // the work-list kernel
   a.direct = a.n_items <= resident ? 1 : 0;
+  a.wave = a.direct ? *grid : std::min(ctx->sms, *grid);
   a.prune = ctx->prune ? 1 : 0;
   return RVH_OK;
 }

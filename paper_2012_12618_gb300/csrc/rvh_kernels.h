@@ -67,6 +67,8 @@ struct FusedArgs {
   int hchunk;
   int pw, hpl;
   int direct;                // 1: one item per CTA, item = blockIdx.x (no work list)
+  int wave;                  // CTA i < wave starts with item i (direct: every CTA, else one per SM); the
+                             // others, and all later rounds, take items wave, wave + 1, ... as they come free
   int prune;                 // 1: staged scoring pass with exact pruning of trials that cannot win
   // [grid * cta_slot_stride(dim, nmax_smem)] FP64 rows, one slot per CTA,
   // used for clusters whose rows fit shared memory (a working set that

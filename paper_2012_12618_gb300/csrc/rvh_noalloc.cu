@@ -140,6 +140,7 @@ extern "C" int rvh_estimate_noalloc(const rvh_frame* f, const rvh_params* p, rvh
   cudaStream_t s = (cudaStream_t)stream;
   const int resident = d->sms * d->occ[dim];
   a.direct = a.n_items <= resident ? 1 : 0;
+  a.wave = a.direct ? a.n_items : d->sms;
   e = rvh::launch_threshold_fill(r->threshold, f->n_clusters, fd.line_model != 0, p->inlier_threshold, s);
   if (e == cudaSuccess && !a.direct) e = rvh::launch_worklist(a, s);
   if (e == cudaSuccess) {
