@@ -92,27 +92,29 @@ __device__ void phase_a_dispatch(int pw, const RV rows, int N, const Smem& S, in
 }
 
 // FP64 rows (a0, a1, a2, w) of a cluster's points.  The 3D model keeps them
-// in global scratch, written once when the cluster is loaded (every 3D trial
-// refines its solve with them); the 2D model computes them when asked (only
-// the winner's inliers, band points and rare refinements need them).
+// in global scratch, written once when the cluster is loaded, with the low
+// parts of the FP32 row (pack_low) in place of w: every 3D trial refines its
+// solve with those, the winner's inliers and band points need the rest.  The
+// 2D model computes its rows when asked (only the winner's inliers, band
+// points and rare refinements need them).
 template <int DIM>
 struct Rows64 {
   const FrameDesc* a;
   int64_t o;
   double4_32a* pre;
-  __device__ __forceinline__ double4_32a at(int j) const {
-    if (DIM == 3) return pre[j];
+  __device__ __forceinline__ double4_32a at(int j) const { return with_w(j, a->dop[o + j]); }
+  // The same row when the point's FP32 cosine-model row, which carries the
+  // Doppler, is at hand.
+  __device__ __forceinline__ double4_32a at(int j, float4 row) const { return with_w(j, DIM == 3 ? row.w : row.z); }
+  __device__ __forceinline__ double4_32a with_w(int j, float w) const {
+    if (DIM == 3) {
+      double4_32a s = pre[j];
+      s.w = (double)w;
+      return s;
+    }
     double t[3];
     row_f64<2>(a->trig, a->az[o + j], 0.0f, t);
-    return make_double4_32a(t[0], t[1], 0.0, (double)a->dop[o + j]);
-  }
-  // The same row when the point's FP32 cosine-model row is at hand: in 2D it
-  // carries the Doppler (row_f32), so only the azimuth is read.
-  __device__ __forceinline__ double4_32a at(int j, float4 row) const {
-    if (DIM == 3) return pre[j];
-    double t[3];
-    row_f64<2>(a->trig, a->az[o + j], 0.0f, t);
-    return make_double4_32a(t[0], t[1], 0.0, (double)row.z);
+    return make_double4_32a(t[0], t[1], 0.0, (double)w);
   }
 };
 
@@ -1108,7 +1110,10 @@ __device__ __forceinline__ void cosine_trial_chunk(const FrameDesc& a, const RV 
     const int q2 = DIM == 3 ? q[2] : q[0];
     const float4 p0 = rows.at(q[0]), p1 = rows.at(q[1]), p2 = rows.at(q2);
     const int qs[3] = {q[0], q[1], q2};
-    auto seed64 = [&](int i) { return R.at(qs[i]); };
+    auto seed64 = [&]() {
+      if constexpr (DIM == 3) return LowSeeds{R.pre, {qs[0], qs[1], qs[2]}};
+      else return [&](int i) { return R.at(qs[i]); };
+    }();
     const float rb = DIM == 3 ? refine_band : __int_as_float(0x7f800000);
     Hyp32 hy = hyp_f32<DIM>(p0, p1, p2, seed64, rb, wmax, a.acc, a.rej, a.tau32);
     if (hy.kind == kHypUndecided) {
@@ -1222,11 +1227,14 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
       const float w = a.dop[o + j];
       const float az = a.az[o + j];
       const float el = DIM == 3 ? a.el[o + j] : 0.0f;
-      rows.put(j, row_f32<DIM>(az, el, w));
+      const float4 row = row_f32<DIM>(az, el, w);
+      rows.put(j, row);
       if (DIM == 3) {
         double a64[3];
         row_f64<DIM>(a.trig, az, el, a64);
-        R.pre[j] = make_double4_32a(a64[0], a64[1], a64[2], (double)w);
+        R.pre[j] = make_double4_32a(
+            a64[0], a64[1], a64[2],
+            pack_low(low_part(a64[0], row.x), low_part(a64[1], row.y), low_part(a64[2], row.z)));
       }
       wm = fmaxf(wm, fabsf(w));
     }
