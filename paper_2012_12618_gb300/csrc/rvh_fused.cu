@@ -194,16 +194,14 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 
 // Upper bound of a normal record's band half-width.
 __device__ __forceinline__ float record_band(float4 hy, float tau_hi, bool line) {
-  return line ? 0x1p-21f * (1.0f + fabsf(hy.x) + fabsf(hy.y) + hy.w) : fmaxf(hy.w - tau_hi, 0.0f) + 0x1p-20f * hy.w;
+  return line ? 0.50001f * (hy.w - hy.z) : fmaxf(hy.w - tau_hi, 0.0f) + 0x1p-20f * hy.w;
 }
 
-// The certain-inlier threshold of a record: |r32| <= tlo is an inlier.  Its
+// The certain-inlier threshold of a record: |r32| <= tlo is an inlier.  The
 // upper threshold thi is tau + b rounded up, so thi - tau bounds the band
-// half-width b; for the line model record_band does, and both thresholds
-// are b away from T distd.
+// half-width b; a line's record, which has no third component, carries tlo there.
 __device__ __forceinline__ float record_tlo(float4 hy, TauPair tau, bool line) {
-  return line ? hy.w * (1.0f - 0x1p-20f) - 2.0f * record_band(hy, tau.hi, true)
-              : __fsub_rd(tau.lo, __fsub_ru(hy.w, tau.hi));
+  return line ? hy.z : __fsub_rd(tau.lo, __fsub_ru(hy.w, tau.hi));
 }
 
 // Where a trial's points can lie, as bins: excess bins 0 .. out of the points
@@ -256,8 +254,10 @@ struct ClusterShared {
   int lo_ok;
   int stop;                   // adaptive trial count: enough trials have run
   double ln_T;                // line model (Alg. 1): the cluster's MAD threshold
-  int sel_digit, sel_k;       // radix select: digit and rank inside it
-  float red4[4][kWarps];      // line model: min / max of azimuth and Doppler
+  int sel_digit, sel_k;       // medians: digit or bin and rank inside it,
+  int sel_hi, sel_n;          // the upper middle's bin, listed keys
+  unsigned long long sel_key[2];  // and the middle keys
+  double ln_min[2], ln_scale[2];  // line model: normalisation of azimuth and Doppler
   unsigned long long runs[2];  // trials run, pairs scored
   unsigned long long scored;   // (trial, point) pairs the scoring pass evaluated
   int nref;                   // 2D trials queued for refinement in the current chunk
@@ -316,7 +316,7 @@ __device__ __forceinline__ void velocity_record(const double v[3], float wmax, T
 // ---- Alg. 1 as printed (line model, 2D): normalised (azimuth, Doppler) points,
 // line fits through two seed points, perpendicular-distance test against the
 // cluster's median absolute deviation.  The FP64 values of each point are
-// kept in its FP64 row slot (x, y, |y - med y|, -), which the 2D cosine
+// kept in its FP64 row slot (x, y, -, -), which the 2D cosine
 // model does not use.
 
 // Alg. 1 point-to-line test in FP64, evaluated as printed: aa = -m, bb = 1,
@@ -327,12 +327,9 @@ __device__ __forceinline__ bool line_in64(double m, double c, double distd, doub
   return fabs(distn / distd) <= thresh;
 }
 
-// FP64 line (m, c, distd) of trial h through its two normalised seed points;
-// false when they share x (no slope).
-__device__ __forceinline__ bool line_hyp64(const FrameDesc& a, const double4_32a* pre, int ci, int h, int N, double v[3]) {
-  int q[3];
-  draw_minimal_set<2>(a.key, a.cluster_base + ci, h, N, q);
-  const double4_32a p0 = pre[q[0]], p1 = pre[q[1]];
+// FP64 line (m, c, distd) through two normalised points; false when they
+// share x (no slope).
+__device__ __forceinline__ bool line_seeds64(const double4_32a& p0, const double4_32a& p1, double v[3]) {
   const double dx = p1.x - p0.x;
   if (dx == 0.0) return false;
   const double m = (p1.y - p0.y) / dx;
@@ -340,6 +337,13 @@ __device__ __forceinline__ bool line_hyp64(const FrameDesc& a, const double4_32a
   v[1] = p0.y - m * p0.x;
   v[2] = sqrt(m * m + 1.0);
   return true;
+}
+
+// The same of trial h, through its two seed points.
+__device__ __forceinline__ bool line_hyp64(const FrameDesc& a, const double4_32a* pre, int ci, int h, int N, double v[3]) {
+  int q[3];
+  draw_minimal_set<2>(a.key, a.cluster_base + ci, h, N, q);
+  return line_seeds64(pre[q[0]], pre[q[1]], v);
 }
 
 // FP32 scoring record of an FP64 line: (-m32, -c32, 0, thi) and tlo, such
@@ -355,37 +359,67 @@ __device__ __forceinline__ Hyp32 line_record(const double v[3], double T) {
   h.refined = 0;
   h.nx = -__double2float_rn(v[0]);
   h.ny = -__double2float_rn(v[1]);
-  h.nz = 0.0f;
   const double td = T * v[2];
   const double am = fabs(v[0]), ac = fabs(v[1]);
   const double b = (0x1p-22 * (1.0 + ac + am + td) + 0x1p-50 * (1.0 + ac + am)) * (1.0 + 0x1p-20);
   const double hi = td * (1.0 + 0x1p-50) + b, lo = td * (1.0 - 0x1p-50) - b;
+  h.kind = kHypNormal;
+  h.thi = __double2float_ru(hi);
+  h.nz = h.tlo = lo >= 0.0 ? __double2float_rd(lo) : -1.0f;
   if (!(hi < 1e30) || !(am < 1e30) || !(ac < 1e30)) {
     h.kind = kHypExactOnly;
     h.thi = __int_as_float(0x7f800000);
-    h.tlo = -1.0f;
-    return h;
+    h.nz = h.tlo = -1.0f;
   }
-  h.thi = __double2float_ru(hi);
-  h.tlo = lo >= 0.0 ? __double2float_rd(lo) : -1.0f;
-  h.kind = kHypNormal;
   return h;
 }
 
-// k-th smallest (0-based, k < N) of the keys |field| of the FP64 point slots
-// (field 1: y, field 2: |y - med y|) as 64-bit patterns of non-negative
-// doubles (monotone as integers; NaN sorts last), by radix digits of 8 bits
-// from the top.  hist: 256 ints of shared memory.  Exact: returns the key.
-template <int FIELD>
-__device__ unsigned long long block_select(const double4_32a* pre, int N, int k, int* hist, ClusterShared& cs) {
+// The same record from the FP32 rows p, q of the two seed points, for seeds
+// at least kLineDx apart in x (kHypUndecided otherwise): FP64 there cost the
+// trial stage a quarter of the line model's time.  With u = 2^-24 the
+// coordinates are within u / 2 of the FP64 ones and the differences dx, dy
+// within u + u|d| <= 2u, so the slope is within dm = 2u (1 + |m|) / |dx| + 4u |m|
+// of the FP64 line's (rcp_approx and one rounding: below 4u).  Against the
+// line through the seeds, r32 carries the points' rounding u (1 + |m|), dm
+// times |x - x0| <= 1, the roundings of c and of two FMAs u (1 + 2|c| + |r|);
+// FP64's own share is 2^-50 (1 + |c| + |m|) as above; distd moves by at most
+// dm and its FP32 evaluation by 2^-21 of it.
+constexpr float kLineDx = 0x1p-12f;
+__device__ __forceinline__ Hyp32 line_record_f32(float4 p, float4 q, TauPair T) {
+  Hyp32 h;
+  h.refined = 0;
+  const float dx = q.x - p.x, dy = q.z - p.z;
+  const float r = rcp_approx(dx);
+  const float m = dy * r, c = fmaf(-m, p.x, p.z);
+  const float am = fabsf(m), ac = fabsf(c);
+  const float dm = kU * (2.01f * (1.0f + am) * fabsf(r) + 4.01f * am);
+  const float sd = sqrt_approx(fmaf(m, m, 1.0f));
+  const float th = T.hi * (sd * (1.0f + 0x1p-20f) + dm) * (1.0f + 0x1p-20f);
+  const float tl = T.lo * (sd * (1.0f - 0x1p-20f) - dm) * (1.0f - 0x1p-20f);
+  const float b = (kU * (2.0f + am + 2.0f * ac + th) + dm) * (1.0f + 0x1p-10f);
+  h.nx = -m;
+  h.ny = -c;
+  h.thi = __fadd_ru(th, b);
+  const float lo = __fsub_rd(tl, b);
+  h.nz = h.tlo = lo >= 0.0f ? lo : -1.0f;
+  h.kind = kHypNormal;
+  if (!(fabsf(dx) >= kLineDx) || !(h.thi < 1e30f)) h.kind = kHypUndecided;
+  return h;
+}
+
+// k-th smallest (0-based, k < N) of N keys: key(j) as 64-bit patterns of
+// non-negative doubles (monotone as integers; NaN sorts last), by radix digits
+// of 8 bits from the top.  hist: 256 ints of shared memory.  Exact: returns
+// the key.
+template <typename Key>
+__device__ __noinline__ unsigned long long block_select(Key key, int N, int k, int* hist, ClusterShared& cs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned long long prefix = 0ull, hmask = 0ull;
   for (int shift = 56; shift >= 0; shift -= 8) {
     hist[tid] = 0;  // kThreads == 256 bins
     __syncthreads();
     for (int j = tid; j < N; j += kThreads) {
-      const double4_32a p = pre[j];
-      const unsigned long long kb = (unsigned long long)__double_as_longlong(fabs(FIELD == 1 ? p.y : p.z));
+      const unsigned long long kb = key(j);
       if ((kb & hmask) == prefix) atomicAdd(&hist[(int)((kb >> shift) & 255ull)], 1);
     }
     __syncthreads();
@@ -418,24 +452,116 @@ __device__ unsigned long long block_select(const double4_32a* pre, int N, int k,
   return prefix;
 }
 
-// Median of the keys (even N: 0.5 * (lower + upper middle)).
-template <int FIELD>
-__device__ double block_median(const double4_32a* pre, int N, int* hist, ClusterShared& cs) {
-  const double hi = __longlong_as_double((long long)block_select<FIELD>(pre, N, N / 2, hist, cs));
-  if (N & 1) return hi;
-  const double lo = __longlong_as_double((long long)block_select<FIELD>(pre, N, N / 2 - 1, hist, cs));
-  return 0.5 * (lo + hi);
+// Bin 0 .. kMedianBins - 1 of a key, monotone in it: the double truncated to
+// FP32 (its high bits; below 2^-126: 0) times the number of bins, NaN and
+// anything from 1 on in the last.
+constexpr int kMedianBins = 1024;
+constexpr int kMedianList = 512;
+__device__ __forceinline__ int median_bin(unsigned long long key) {
+  const int hi = (int)(key >> 32);
+  if (hi < 0x38100000) return 0;
+  if (hi >= 0x3ff00000) return kMedianBins - 1;
+  const float f = __int_as_float(((hi - 0x38000000) << 3) | (int)((unsigned)key >> 29));
+  return (int)(f * (float)kMedianBins);
+}
+
+// Median of N keys (even N: 0.5 * (lower + upper middle)), exact: a histogram
+// of kMedianBins even bins over [0, 1] finds the bins of the two middle
+// ranks, whose few keys are ranked against each other; more than kMedianList
+// keys in them (few distinct values) go to the radix select.  Two passes over
+// the keys instead of eight per middle: the radix selects over global memory
+// took 44% of the line model's time (dense2d 0.69 -> 0.47 ms).  hist:
+// kMedianBins ints, list: kMedianList keys of shared memory.
+template <typename Key>
+__device__ __forceinline__ double block_median(Key key, int N, int* hist, unsigned long long* list,
+                                               ClusterShared& cs) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int k1 = N >> 1, k0 = (N & 1) ? k1 : k1 - 1;
+  constexpr int kPer = kMedianBins / kThreads;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) hist[tid + i * kThreads] = 0;
+  if (tid == 0) cs.sel_n = 0;
+  __syncthreads();
+  for (int j = tid; j < N; j += kThreads) atomicAdd(&hist[median_bin(key(j))], 1);
+  __syncthreads();
+  int c[kPer], tot = 0;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    c[i] = hist[kPer * tid + i];
+    tot += c[i];
+  }
+  int incl = tot;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += t;
+  }
+  if (lane == 31) cs.red_i[warp] = incl;
+  __syncthreads();
+  int below = incl - tot;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) below += w < warp ? cs.red_i[w] : 0;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    if (below <= k0 && k0 < below + c[i]) {
+      cs.sel_digit = kPer * tid + i;
+      cs.sel_k = k0 - below;  // rank of the lower middle among the listed keys
+    }
+    if (below <= k1 && k1 < below + c[i]) cs.sel_hi = kPer * tid + i;
+    below += c[i];
+  }
+  __syncthreads();
+  const int b0 = cs.sel_digit, b1 = cs.sel_hi;  // no key lies in a bin between them
+  for (int j = tid; j < N; j += kThreads) {
+    const unsigned long long kb = key(j);
+    const int b = median_bin(kb);
+    if (b == b0 || b == b1) {
+      const int pos = atomicAdd(&cs.sel_n, 1);
+      if (pos < kMedianList) list[pos] = kb;
+    }
+  }
+  __syncthreads();
+  const int m = cs.sel_n, r0 = cs.sel_k;
+  if (m > kMedianList) {
+    const double hi = __longlong_as_double((long long)block_select(key, N, k1, hist, cs));
+    if (N & 1) return hi;
+    const double lo = __longlong_as_double((long long)block_select(key, N, k0, hist, cs));
+    return 0.5 * (lo + hi);
+  }
+  for (int i = tid; i < m; i += kThreads) {
+    const unsigned long long ki = list[i];
+    int rank = 0;
+    for (int t = 0; t < m; ++t) rank += list[t] < ki || (list[t] == ki && t < i) ? 1 : 0;
+    if (rank == r0) cs.sel_key[0] = ki;
+    if (rank == r0 + (k1 - k0)) cs.sel_key[1] = ki;
+  }
+  __syncthreads();
+  const double lo = __longlong_as_double((long long)cs.sel_key[0]);
+  const double hi = __longlong_as_double((long long)cs.sel_key[1]);
+  return (N & 1) ? hi : 0.5 * (lo + hi);
+}
+
+// Bytes of the trial area of shared memory: hchunk trials, and at least the
+// final reduction (up to 9 sums per thread).
+__host__ __device__ constexpr size_t trial_area_bytes(int hchunk) {
+  const size_t trials = (size_t)hchunk * (sizeof(float4) + sizeof(float) + sizeof(int) + sizeof(uint16_t)) +
+                        (((size_t)hchunk + 15) & ~(size_t)15);
+  const size_t reduction = (size_t)9 * kThreads * sizeof(double);
+  return trials > reduction ? trials : reduction;
 }
 
 // The line model's rows stage: min / max of azimuth and Doppler, normalised
 // FP64 points into the FP64 slots and FP32 rows (x, 1, y) into the scoring
 // rows, then the MAD threshold into cs.ln_T.  Normalisation (the paper's
 // normalize(), undefined there): min-max scaling, x = (t - t_min) *
-// (1 / (t_max - t_min)), 0 when the range is empty.  Out of line: runs once
-// per cluster.
+// (1 / (t_max - t_min)), 0 when the range is empty.  The trial area of shared
+// memory is free at this point: it holds the medians' histogram and list, and
+// the FP64 Dopplers of as many points as fit the rest (2432 with the default
+// sizes; larger clusters read them back from their slots).  Out of line:
+// runs once per cluster.
 template <typename RV>
 __device__ __noinline__ void line_rows_and_threshold(const FrameDesc& a, const RV rows, double4_32a* pre, int64_t o,
-                                                     int N, int* hist, ClusterShared& cs) {
+                                                     int N, const Smem& S, int hchunk, ClusterShared& cs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float inf = __int_as_float(0x7f800000);
   float m4[4] = {inf, inf, inf, inf};  // min t, -max t, min v, -max v
@@ -448,34 +574,42 @@ __device__ __noinline__ void line_rows_and_threshold(const FrameDesc& a, const R
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) m4[i] = fminf(m4[i], __shfl_xor_sync(0xffffffffu, m4[i], d));
-    if (lane == 0) cs.red4[i][warp] = m4[i];
+    const int r = __reduce_min_sync(0xffffffffu, float_order(m4[i]));
+    if (lane == 0) cs.red_d[i][warp] = r;
   }
   __syncthreads();
+  if (tid < 2) {  // azimuth, Doppler
+    int lo = cs.red_d[2 * tid][0], hi = cs.red_d[2 * tid + 1][0];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float r = cs.red4[i][0];
-#pragma unroll
-    for (int w = 1; w < kWarps; ++w) r = fminf(r, cs.red4[i][w]);
-    m4[i] = r;
+    for (int w = 1; w < kWarps; ++w) {
+      lo = min(lo, cs.red_d[2 * tid][w]);
+      hi = min(hi, cs.red_d[2 * tid + 1][w]);
+    }
+    const double l = (double)order_float(lo), h = -(double)order_float(hi);
+    cs.ln_min[tid] = l;
+    cs.ln_scale[tid] = h > l ? 1.0 / (h - l) : 0.0;
   }
-  const double tmin = (double)m4[0], tmax = -(double)m4[1], vmin = (double)m4[2], vmax = -(double)m4[3];
-  const double rt = tmax > tmin ? 1.0 / (tmax - tmin) : 0.0;
-  const double rv = vmax > vmin ? 1.0 / (vmax - vmin) : 0.0;
+  __syncthreads();
+  const double tmin = cs.ln_min[0], vmin = cs.ln_min[1], rt = cs.ln_scale[0], rv = cs.ln_scale[1];
+  int* hist = reinterpret_cast<int*>(S.hyp);
+  unsigned long long* list = reinterpret_cast<unsigned long long*>(hist + kMedianBins);
+  double* sy = reinterpret_cast<double*>(list + kMedianList);
+  const bool in_smem =
+      N <= (int)((trial_area_bytes(hchunk) - kMedianBins * sizeof(int)) / sizeof(double)) - kMedianList;
   for (int j = tid; j < N; j += kThreads) {
-    const double x = ((double)a.az[o + j] - tmin) * rt;
+    const float az = a.az[o + j];
+    const double x = ((double)az - tmin) * rt;
     const double y = ((double)a.dop[o + j] - vmin) * rv;
     pre[j] = make_double4_32a(x, y, 0.0, 0.0);
-    const float y32 = __double2float_rn(y);
-    rows.put(j, make_float4(__double2float_rn(x), 1.0f, y32, a.az[o + j]));
+    rows.put(j, make_float4(__double2float_rn(x), 1.0f, __double2float_rn(y), az));
+    if (in_smem) sy[j] = y;
   }
-  __syncthreads();
-  // Eq. eq:MAD read as the median absolute deviation of the normalised Doppler
-  const double med = block_median<1>(pre, N, hist, cs);
-  for (int j = tid; j < N; j += kThreads) pre[j].z = fabs(pre[j].y - med);
-  __syncthreads();
-  const double T = block_median<2>(pre, N, hist, cs);
+  // Eq. eq:MAD read as the median absolute deviation of the normalised
+  // Doppler; each thread reads the keys it wrote
+  auto y_at = [&](int j) { return in_smem ? sy[j] : pre[j].y; };
+  auto bits = [](double d) { return (unsigned long long)__double_as_longlong(fabs(d)); };
+  const double med = block_median([&](int j) { return bits(y_at(j)); }, N, hist, list, cs);
+  const double T = block_median([&](int j) { return bits(y_at(j) - med); }, N, hist, list, cs);
   if (tid == 0) cs.ln_T = T;
   __syncthreads();
 }
@@ -1241,7 +1375,7 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
   };
   if constexpr (EXT && DIM == 2) {
     if (a.line_model) {
-      line_rows_and_threshold<RV>(a, rows, R.pre, o, N, S.U, cs);
+      line_rows_and_threshold<RV>(a, rows, R.pre, o, N, S, hchunk, cs);
       if (tid == 0 && a.threshold) a.threshold[ci] = cs.ln_T;  // the API wrote NaN before
     } else {
       cosine_rows();
@@ -1276,21 +1410,24 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
     };
     if constexpr (EXT && DIM == 2) {
       if (a.line_model) {
+        const TauPair T = {__double2float_rd(cs.ln_T), __double2float_ru(cs.ln_T)};
         for (int hl = tid; hl < nh; hl += kThreads) {
-          // Alg. 1: the line through the two normalised seed points, in FP64
-          double v[3];
-          Hyp32 hy;
-          if (line_hyp64(a, R.pre, ci, hc0 + hl, N, v)) {
-            hy = line_record(v, cs.ln_T);
-          } else {
-            hy.kind = kHypRejected;
-            hy.nx = hy.ny = hy.nz = 0.0f;
-            hy.tlo = -1.0f;
-            hy.thi = 0.0f;
+          // Alg. 1: the line through the two normalised seed points
+          int q[3];
+          draw_minimal_set<2>(a.key, a.cluster_base + ci, hc0 + hl, N, q);
+          Hyp32 hy = line_record_f32(rows.at(q[0]), rows.at(q[1]), T);
+          if (hy.kind == kHypUndecided) {
+            double v[3];
+            if (line_seeds64(R.pre[q[0]], R.pre[q[1]], v)) {
+              hy = line_record(v, cs.ln_T);
+            } else {
+              hy.kind = kHypRejected;
+              hy.nx = hy.ny = hy.nz = 0.0f;
+            }
           }
           if (hy.kind == kHypExactOnly) ++n_fp64;
           S.hyp[hl] = make_float4(hy.nx, hy.ny, hy.nz, hy.kind == kHypRejected ? __int_as_float(0x7fc00000) : hy.thi);
-                S.kind[hl] = (int8_t)hy.kind;
+          S.kind[hl] = (int8_t)hy.kind;
           S.U[hl] = hy.kind == kHypRejected ? -1 : (hy.kind == kHypExactOnly ? N : 0);
         }
       } else {
@@ -1605,11 +1742,7 @@ __global__ void worklist_kernel(const __grid_constant__ FusedArgs a) {
 }
 
 size_t fused_smem_bytes(int nmax_smem, int hchunk) {
-  // the trial area also holds the final reduction (up to 9 sums per thread)
-  const size_t trials = (size_t)hchunk * (sizeof(float4) + sizeof(float) + sizeof(int) + sizeof(uint16_t)) +
-                        (((size_t)hchunk + 15) & ~(size_t)15);
-  const size_t reduction = (size_t)9 * kThreads * sizeof(double);
-  return (size_t)((nmax_smem + 31) & ~31) * sizeof(float4) + (trials > reduction ? trials : reduction);
+  return (size_t)((nmax_smem + 31) & ~31) * sizeof(float4) + trial_area_bytes(hchunk);
 }
 
 cudaError_t launch_worklist(const FusedArgs& a, cudaStream_t s) {
