@@ -168,8 +168,9 @@ __device__ __forceinline__ int excess_bin(float x) {
 }
 
 // The cluster's directions a: range of t = a1 / a0, 1 / min a0 and max|a2|;
-// tan_ok = 0 (some a0 not safely positive, or rows that are no directions)
-// leaves the interval test out.
+// tan_ok = 0 (some a0 not safely positive) leaves the interval test out.
+// The line model's rows (x, 1, y) have residuals of the same form with a =
+// (1, x): t = x in [0, 1], a0 = 1, and the components of d change places.
 struct DirRange {
   float t0, tinv, tabs, a0inv, zmax;
   int tan_ok;
@@ -177,6 +178,11 @@ struct DirRange {
 
 __device__ __forceinline__ int tan_bin(const DirRange& g, float t) {
   return min(max(__float2int_rd((t - g.t0) * g.tinv), 0), kTanBins - 1);
+}
+
+template <typename Row>
+__device__ __forceinline__ float row_tan(const Row& p, bool line) {
+  return line ? p.x : p.y * rcp_approx(p.x);
 }
 
 // floats as integers of the same order, and back
@@ -217,11 +223,12 @@ template <int DIM>
 __device__ __forceinline__ HoldRange hold_range(const DirRange& g, float4 lead, float lead_band, bool line, float4 hy) {
   // thi_h covers tau and the velocity error of h; 2 lead_band covers the
   // lead's velocity and residuals
-  const float dx = hy.x - lead.x, dy = hy.y - lead.y, dz = DIM == 3 ? hy.z - lead.z : 0.0f;
+  const float d0 = hy.x - lead.x, d1 = hy.y - lead.y, dz = DIM == 3 ? hy.z - lead.z : 0.0f;
+  const float dx = line ? d1 : d0, dy = line ? d0 : d1;
   const float ax = fabsf(dx), ay = fabsf(dy), az = DIM == 3 ? g.zmax * fabsf(dz) : 0.0f;
   const float slack = 2.0f * lead_band + 4e-6f * (ax + ay + fabsf(dz));
-  // max|a.d|: unit directions, or (x, 1) with x in [0, 1] for the line model
-  const float reach = line ? ax + ay : sqrt_approx(fmaf(dx, dx, dy * dy)) + az;
+  // max|a.d|: unit directions, or the ends of x's range for the line model
+  const float reach = line ? fmaxf(ax, fabsf(dx + dy)) : sqrt_approx(fmaf(dx, dx, dy * dy)) + az;
   const uint32_t out = (uint32_t)excess_bin((hy.w + reach + slack) * 1.0001f - lead.w);
   uint32_t lo = 0u, hi = kTanBins;
   if (g.tan_ok) {
@@ -1015,14 +1022,14 @@ constexpr int kStageMaxPoints = 32767;  // points are counted in 16-bit halves
 // warp's part into cs.red_d; the caller's next barrier is followed by
 // direction_range_finish.
 template <int DIM, typename RV>
-__device__ __forceinline__ void direction_range(const RV rows, int N, ClusterShared& cs) {
+__device__ __forceinline__ void direction_range(const RV rows, int N, bool line, ClusterShared& cs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float inf = __int_as_float(0x7f800000);
   float a0 = inf, t0 = inf, t1 = -inf, z = 0.0f;
   for (int j = tid; j < N; j += kThreads) {
     const float4 p = rows.at(j);
-    const float t = p.y * rcp_approx(p.x);
-    a0 = fminf(a0, p.x);
+    const float t = row_tan(p, line);
+    a0 = fminf(a0, line ? p.y : p.x);
     t0 = fminf(t0, t);
     t1 = fmaxf(t1, t);
     if (DIM == 3) z = fmaxf(z, fabsf(p.z));
@@ -1039,7 +1046,7 @@ __device__ __forceinline__ void direction_range(const RV rows, int N, ClusterSha
 }
 
 template <int DIM>
-__device__ __forceinline__ void direction_range_finish(bool line, ClusterShared& cs) {
+__device__ __forceinline__ void direction_range_finish(ClusterShared& cs) {
   if (threadIdx.x != 0) return;
   int r[4];
 #pragma unroll
@@ -1055,7 +1062,7 @@ __device__ __forceinline__ void direction_range_finish(bool line, ClusterShared&
   cs.dir.tabs = fmaxf(fabsf(t0), fabsf(t1));
   cs.dir.a0inv = rcp_approx(a0) * kRcpUp;
   cs.dir.zmax = DIM == 3 ? order_float(r[3]) : 0.0f;
-  cs.dir.tan_ok = !line && a0 > 1e-3f && a0 < 2.0f;
+  cs.dir.tan_ok = a0 > 1e-3f && a0 < 2.0f;
 }
 
 // Scores the chunk's normal trials in stages.  After the first stage the
@@ -1124,7 +1131,7 @@ __device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, co
       if (q >= q0) {
         const unsigned one = (q < e1 || (q >= e2 && q < e3)) ? 1u : 1u << 16;
         if (r <= lw.w)
-          atomicAdd(&cs.lead_in[(q < e2 ? 0 : kTanBins + 1) + tan_bin(dir, p.y * rcp_approx(p.x))], one);
+          atomicAdd(&cs.lead_in[(q < e2 ? 0 : kTanBins + 1) + tan_bin(dir, row_tan(p, line))], one);
         else if (r > lw.w)  // NaN: held by no trial
           atomicAdd(&cs.lead_out[(q < e2 ? 0 : kExcessBins) + excess_bin(r - lw.w)], one);
       }
@@ -1393,9 +1400,10 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
     cs.nref = 0;
   }
   const bool may_stage = prune && pw == 1 && N >= kStageMinPoints && N <= kStageMaxPoints;
-  if (may_stage) direction_range<DIM>(rows, N, cs);
+  const bool line = EXT && DIM == 2 && a.line_model;
+  if (may_stage) direction_range<DIM>(rows, N, line, cs);
   const float wmax = block_max_float(wm, cs.red_f);  // its barrier also orders the row writes
-  if (may_stage) direction_range_finish<DIM>(EXT && DIM == 2 && a.line_model, cs);
+  if (may_stage) direction_range_finish<DIM>(cs);
   unsigned long long n_fp64 = 0, n_cand = 0, n_ref = 0, n_scored = 0;
   stage_done(0);
 
@@ -1444,7 +1452,7 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
     // becomes the lead if its key beats it
     auto count_trial = [&](int c) {
       const float4 hy = S.hyp[c];
-      const float htlo = record_tlo(hy, a.tau32, EXT && DIM == 2 && a.line_model);
+      const float htlo = record_tlo(hy, a.tau32, line);
       int B = 0;
       const int C = exact_count_block<DIM, RV, EXT>(a, rows, R, ci, hc0 + c, N, hy, htlo, cs, &B);
       ++n_cand;
@@ -1534,7 +1542,7 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
   // whose FP64 velocity was computed when it was counted) and the normal
   // equations over its inliers.
   const float4 win = cs.win;
-  const float wtlo = record_tlo(win, a.tau32, EXT && DIM == 2 && a.line_model);
+  const float wtlo = record_tlo(win, a.tau32, line);
   const double v64[3] = {cs.win_v64[0], cs.win_v64[1], cs.win_v64[2]};
   constexpr int NS = DIM == 2 ? 5 : 9;
   int n_in = mask_and_sums<DIM, RV, EXT>(a, rows, R, o, N, win, wtlo, v64, S, cs, false, nullptr);
