@@ -25,9 +25,9 @@
 // neighbour, walk alone (batched loads) when their neighbourhood is small
 // and with the whole warp (coalesced tiles, ballots) when it is large.  Then
 // a lock-free union-find over core-core neighbour pairs on sorted positions:
-// a near-neighbour linking pass and a compression first, a root recorded
-// per bucket, and a full per-thread pass that skips buckets already in the
-// point's set; it links the larger root under the smaller.  An atomic
+// a near-neighbour linking pass within blocks first, a root recorded
+// per bucket, and a full pass, eight lanes per point, that skips buckets
+// already in the point's set; it links the larger root under the smaller.  An atomic
 // minimum per component gives its smallest core index; a device-wide scan
 // numbers the clusters.  The CSR:
 // per-cluster counts, offsets by a scan, placement, and a shared-memory sort
@@ -64,6 +64,7 @@ struct ClusterArgs {
   int2* bslot;         // [n] (bucket, slot within the bucket) of each point
   float4* sfeat;       // [n] features in sorted order, zero-padded to four
   int* sidx;           // [n] original index of each sorted position
+  uint32_t* sbkt;      // [n] bucket of each sorted position
   uint8_t* score;      // [n] core flag by sorted position
   uint8_t* core;       // [n] core flag by original index
   int* parent;         // [n] union-find over sorted positions
@@ -117,7 +118,7 @@ __device__ __forceinline__ bool is_neighbour(const ClusterArgs& a, const float4&
   return s64 <= a.eps2;  // NaN: false
 }
 
-struct Cell {
+struct Cell {  // cell coordinates, or their bits that make the bucket: neighbours are taken modulo the table
   int x, y, z;
 };
 
@@ -130,6 +131,13 @@ __device__ __forceinline__ Cell cell_of(const ClusterArgs& a, const float4& f) {
 
 __device__ __forceinline__ uint32_t bucket_of(const ClusterArgs& a, const Cell& c) {
   return row_bucket(a, c.y, c.z) | ((uint32_t)c.x & a.xmask);
+}
+
+// The cell of a sorted position, from its bucket (forming it from the features
+// again takes FP64 instructions, which are slow on this GPU).
+__device__ __forceinline__ Cell cell_at(const ClusterArgs& a, int64_t s) {
+  const uint32_t b = a.sbkt[s];
+  return Cell{(int)(b & a.xmask), (int)(b >> a.ysh & a.ymask), (int)(b >> a.zsh & a.zmask)};
 }
 
 // Calls span(begin, end) for the sorted-position ranges, cut at limit, that
@@ -172,22 +180,6 @@ __device__ __forceinline__ bool for_chunks(const ClusterArgs& a, const Cell& c, 
   });
 }
 
-// Calls bucket(b) for the 3^g distinct buckets around cell c, the cell's own
-// row first, until bucket returns false.
-template <int DIM, typename Bucket>
-__device__ __forceinline__ bool for_buckets(const ClusterArgs& a, const Cell& c, Bucket bucket) {
-  constexpr int G = DIM < 3 ? DIM : 3;
-  constexpr int RY = G > 1 ? 1 : 0, RZ = G > 2 ? 1 : 0;
-  for (int iz = 0; iz <= 2 * RZ; ++iz)
-    for (int iy = 0; iy <= 2 * RY; ++iy) {
-      const int dz = iz == 2 ? -1 : iz, dy = iy == 2 ? -1 : iy;
-      const uint32_t row = row_bucket(a, c.y + dy, c.z + dz);
-      for (int dx = -1; dx <= 1; ++dx)
-        if (!bucket(row + ((uint32_t)(c.x + dx) & a.xmask))) return false;
-    }
-  return true;
-}
-
 // the number of candidates of cell c (the sizes of its ranges)
 template <int DIM>
 __device__ __forceinline__ int cand_count(const ClusterArgs& a, const Cell& c) {
@@ -226,18 +218,13 @@ __device__ __forceinline__ Cell shfl_cell(const Cell& c, int src) {
   return Cell{__shfl_sync(kFull, c.x, src), __shfl_sync(kFull, c.y, src), __shfl_sync(kFull, c.z, src)};
 }
 
-template <int DIM>
-__device__ __forceinline__ uint32_t point_bucket(const ClusterArgs& a, const float4& f) {
-  return bucket_of(a, cell_of<DIM>(a, f));
-}
-
 // bucket and slot of every point (the slot order within a bucket is
 // arbitrary; no result depends on it)
 template <int DIM>
 __global__ void k_grid(ClusterArgs a) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.n) return;
-  const uint32_t b = point_bucket<DIM>(a, load_feat<DIM>(a.feat + i * DIM));
+  const uint32_t b = bucket_of(a, cell_of<DIM>(a, load_feat<DIM>(a.feat + i * DIM)));
   a.bslot[i] = make_int2((int)b, atomicAdd(&a.count[b], 1));
 }
 
@@ -256,6 +243,7 @@ __global__ void k_scatter(ClusterArgs a) {
   const int pos = a.start[bs.x] + bs.y;
   a.sfeat[pos] = load_feat<DIM>(a.feat + i * DIM);
   a.sidx[pos] = (int)i;
+  a.sbkt[pos] = (uint32_t)bs.x;
 }
 
 // Neighbour counts (stopping at min_pts), one thread per sorted position.
@@ -271,10 +259,10 @@ __global__ void k_core(ClusterArgs a) {
   if (s - lane >= a.n) return;  // the whole warp
   const bool live = s < a.n;
   const float4 fp = a.sfeat[live ? s : a.n - 1];
-  const Cell c = cell_of<DIM>(a, fp);
+  const Cell c = cell_at(a, live ? s : a.n - 1);
   int count = 0;
   if (live) {
-    const uint32_t bk = bucket_of(a, c);
+    const uint32_t bk = a.sbkt[s];
     const int b = a.start[bk], e = min(a.start[bk + 1], b + kOwnCap);
     for (int t0 = b; t0 < e && count < a.min_pts; t0 += kChunk) {
       float4 fq[kChunk];
@@ -367,111 +355,200 @@ __device__ __forceinline__ bool uf_union(const ClusterArgs& a, int& rp, int pt) 
 }
 
 // Joins every core point with its core neighbours at lower sorted positions
-// (each core-core pair once), one thread per point, bucket by bucket.  rp is
-// the point's root as last seen and alias the last ancestor it merged: both
-// stay in its set for good.  A bucket whose core points all had root rb
-// after the compression needs no look at all when rb is rp or alias, and
-// otherwise only its first core neighbour: one link to rb joins them all.
-// A bucket with mixed roots is walked candidate by candidate.
-template <int DIM>
+// (each core-core pair once), kUG lanes per point.  rp is the point's root as
+// last seen (the smallest any lane saw) and alias the last ancestor a lane
+// merged: both stay in its set for good.  A bucket whose core points all had
+// root rb when the bucket roots were taken needs no look at all when rb is rp,
+// and otherwise only its first core neighbour: one link to rb joins them all.
+// A bucket with mixed roots is walked candidate by candidate.  The roots of
+// kUG buckets are looked at together, and the lanes share a bucket's
+// candidates.  The pass runs twice: first for every kSample-th position, a
+// warp each, which joins nearly all cells that touch; then, after the bucket
+// roots are taken anew, for the others, which find most of their buckets
+// already in their set.  What bounds it are chains of dependent L2 loads, so
+// lanes that follow different points of a warp cost each other their time:
+// on the 106 k-point scene 110 us with a thread per point, 120 with eight
+// lanes, 82 + 44 sampled (eight lanes both), and the whole call 325 -> 270 us
+// as it stands (32 and 8 lanes, every 8th position: 291).
+constexpr int kUGSampled = 32, kUGRest = 16;
+constexpr int kSample = 16;
+template <int DIM, bool SAMPLED>
 __global__ void k_union(ClusterArgs a) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= a.n || !a.score[s]) return;
+  constexpr int kUG = SAMPLED ? kUGSampled : kUGRest;
+  constexpr unsigned kGroup = kUG == 32 ? kFull : (1u << kUG) - 1u;
+  constexpr int G = DIM < 3 ? DIM : 3;
+  constexpr int NX = 3, NY = G > 1 ? 3 : 1, NZ = G > 2 ? 3 : 1, NC = NX * NY * NZ;
+  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t s = SAMPLED ? gid / kUG * kSample : gid / kUG;
+  const int lane = threadIdx.x & 31, sub = lane & (kUG - 1), lead = lane & ~(kUG - 1);
+  const unsigned group = kGroup << lead;
+  if (s >= a.n || !a.score[s] || (!SAMPLED && s % kSample == 0)) return;  // the whole group
   const float4 fp = a.sfeat[s];
-  int rp = uf_find(a.parent, (int)s);
-  int alias = rp;
-  for_buckets<DIM>(a, cell_of<DIM>(a, fp), [&](uint32_t b) {
-    const int rb = a.broot[b];
-    if (rb == kNoCore || rb == rp || rb == alias) return true;
-    const int lo = a.start[b], hi = min(a.start[b + 1], (int)s);
-    if (rb >= 0) {
-      bool found = false;
-      for (int t0 = lo; t0 < hi && !found; t0 += kChunk) {
-        bool sc[kChunk];
-        float4 fq[kChunk];
-#pragma unroll
-        for (int u = 0; u < kChunk; ++u) {
-          sc[u] = a.score[min(t0 + u, hi - 1)];
-          fq[u] = a.sfeat[min(t0 + u, hi - 1)];
-        }
-#pragma unroll
-        for (int u = 0; u < kChunk; ++u)
-          if (t0 + u < hi && sc[u] && is_neighbour<DIM>(a, fp, fq[u])) found = true;
-      }
-      if (found) {
-        if (!uf_union(a, rp, rb)) return false;
-        alias = rb;
-      }
-      return true;
+  const Cell c = cell_at(a, s);
+  int rp = 0;
+  if (sub == 0) rp = uf_find(a.parent, (int)s);
+  rp = __shfl_sync(group, rp, lead);
+  for (int c0 = 0; c0 < NC; c0 += kUG) {
+    const int i = c0 + sub;
+    uint32_t bk = 0;
+    int rb = kNoCore;
+    if (i < NC) {
+      // the cell's own row first
+      const int ix = i % 3, iy = (i / 3) % NY, iz = i / (3 * NY);
+      const int dy = iy == 2 ? -1 : iy, dz = iz == 2 ? -1 : iz;
+      bk = row_bucket(a, c.y + dy, c.z + dz) + ((uint32_t)(c.x + ix - 1) & a.xmask);
+      rb = a.broot[bk];
     }
-    for (int t0 = lo; t0 < hi; t0 += kChunk) {
-      bool sc[kChunk];
-      int tag[kChunk];
+    unsigned todo = __ballot_sync(group, rb != kNoCore && rb != rp) >> lead & kGroup;
+    for (; todo; todo &= todo - 1u) {
+      const int src = lead + __ffs(todo) - 1;
+      const uint32_t b = __shfl_sync(group, bk, src);
+      const int r = __shfl_sync(group, rb, src);
+      if (r == rp) continue;
+      const int lo = a.start[b], hi = min(a.start[b + 1], (int)s);
+      bool ok = true;
+      if (r >= 0) {
+        bool found = false;
+        for (int t0 = lo; t0 < hi && !found; t0 += kUG * kChunk / 2) {
+          bool mine = false;
 #pragma unroll
-      for (int u = 0; u < kChunk; ++u) {
-        sc[u] = a.score[min(t0 + u, hi - 1)];
-        tag[u] = __ldcg(&a.parent[min(t0 + u, hi - 1)]);
-      }
-#pragma unroll
-      for (int u = 0; u < kChunk; ++u)
-        if (t0 + u < hi && sc[u] && tag[u] != rp && tag[u] != alias && is_neighbour<DIM>(a, fp, a.sfeat[t0 + u])) {
-          if (!uf_union(a, rp, tag[u])) return false;
-          alias = tag[u];
+          for (int u = 0; u < kChunk / 2; ++u) {
+            const int t = t0 + u * kUG + sub, tc = min(t, hi - 1);
+            const bool sc = a.score[tc];
+            const float4 fq = a.sfeat[tc];
+            if (t < hi && sc && is_neighbour<DIM>(a, fp, fq)) mine = true;
+          }
+          found = __any_sync(group, mine);
         }
+        if (found && sub == 0) ok = uf_union(a, rp, r);
+      } else {
+        int alias = rp;
+        for (int t0 = lo; t0 < hi && ok; t0 += kUG * kChunk / 2) {
+#pragma unroll
+          for (int u = 0; u < kChunk / 2; ++u) {
+            const int t = t0 + u * kUG + sub, tc = min(t, hi - 1);
+            const bool sc = a.score[tc];
+            const int tag = __ldcg(&a.parent[tc]);
+            if (t < hi && sc && tag != rp && tag != alias && is_neighbour<DIM>(a, fp, a.sfeat[tc])) {
+              ok = ok && uf_union(a, rp, tag);
+              alias = tag;
+            }
+          }
+        }
+      }
+      if (!__all_sync(group, ok)) return;  // the retry cap ran out: flagged
+      // every lane's rp is an ancestor of the point; the smallest is nearest the root
+#pragma unroll
+      for (int d = kUG / 2; d > 0; d >>= 1) rp = min(rp, __shfl_xor_sync(group, rp, d));
     }
-    return true;
-  });
+  }
 }
 
 // A cheap first linking pass (the sampling idea of Afforest, Sutton et al.,
-// IPDPS'18): every core point joins the core neighbours among the kNear
-// positions just before it, mostly points of its own cell.  After k_compress
-// most points of a dense cell share one root, and the full walk of k_union
-// then meets pairs whose parent already is the root.  Any subset of the
-// core-core edges may be linked early: the components are the same.
-constexpr int kNear = 4;
+// IPDPS'18): within a block of kLT consecutive sorted positions, mostly points
+// of the same few cells, every core point joins the core neighbours among the
+// kNear positions just before it.  The components of those links are found
+// in shared memory: every point takes the smallest label among its links and
+// the label of that label until none changes, and parent is set to it, so the
+// forest starts with trees of depth one.  (As global unions the same links
+// took 36 us on the 106 k-point scene, long chains of compare-and-swaps, and
+// a compression pass 5 us; this pass takes 9 us.)  Any subset of the core-core
+// edges may be linked early: the components are the same.  Labels only
+// decrease along links, so a forest stopped at the round cap is still valid.
+constexpr int kNear = 8;
+constexpr int kLT = 512;
+constexpr int kLinkRounds = 64;
 template <int DIM>
-__global__ void k_union_near(ClusterArgs a) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= a.n || !a.score[s]) return;
-  const float4 fp = a.sfeat[s];
-  int rp = uf_find(a.parent, (int)s);
-  const int64_t lo = s > kNear ? s - kNear : 0;
-  for (int64_t t = s - 1; t >= lo; --t)
-    if (a.score[t] && is_neighbour<DIM>(a, fp, a.sfeat[t]))
-      if (!uf_union(a, rp, __ldcg(&a.parent[t]))) return;
-}
-
-// points every core point's parent at its root (no links meanwhile)
-__global__ void k_compress(ClusterArgs a) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= a.n || !a.score[s]) return;
-  a.parent[s] = uf_find(a.parent, (int)s);
+__global__ void __launch_bounds__(kLT) k_link_blocks(ClusterArgs a) {
+  __shared__ float4 f[kLT];
+  __shared__ int label[kLT];
+  const int t = threadIdx.x;
+  const int64_t s = (int64_t)blockIdx.x * kLT + t;
+  const bool core = s < a.n && a.score[s];
+  float4 fp = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (core) fp = a.sfeat[s];
+  f[t] = fp;
+  label[t] = core ? t : -1;
+  __syncthreads();
+  unsigned link = 0u;
+  if (core) {
+#pragma unroll
+    for (int k = 1; k <= kNear; ++k)
+      if (t >= k && label[t - k] >= 0 && is_neighbour<DIM>(a, fp, f[t - k])) link |= 1u << k;
+  }
+  __syncthreads();
+  for (int r = 0; r < kLinkRounds; ++r) {
+    int m = core ? label[t] : 0;
+    const int was = m;
+    int most = m;
+    if (core) {
+      for (unsigned l = link; l; l &= l - 1u) {
+        const int v = label[t - (__ffs(l) - 1)];
+        m = min(m, v);
+        most = max(most, v);
+      }
+      m = min(m, label[m]);
+    }
+    __syncthreads();
+    // the smaller label goes to both ends of each link and to the entries of
+    // the labels it replaces
+    if (core && m < was) {
+      atomicMin(&label[was], m);
+      atomicMin(&label[t], m);
+    }
+    if (core && m < most) {
+      for (unsigned l = link; l; l &= l - 1u) {
+        const int e = t - (__ffs(l) - 1), v = label[e];
+        if (v > m) {
+          atomicMin(&label[v], m);
+          atomicMin(&label[e], m);
+        }
+      }
+    }
+    if (!__syncthreads_or(core && m < most)) break;
+  }
+  if (core) a.parent[s] = (int)((int64_t)blockIdx.x * kLT) + label[t];
 }
 
 // Per bucket, the root its core points share, or -1 (mixed): each core
 // point walks to its root (no links meanwhile; parents read here are all
-// ancestors), points its own parent there, and marks its bucket.
-template <int DIM>
+// ancestors), points its own parent there, and the lanes of a bucket mark it
+// together.
 __global__ void k_bucket_roots(ClusterArgs a) {
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= a.n || !a.score[s]) return;
+  const bool core = s < a.n && a.score[s];
+  const unsigned act = __ballot_sync(kFull, core);
+  if (!core) return;
   int x = (int)s, p = __ldcg(&a.parent[x]);
   while (p != x) {
     x = p;
     p = __ldcg(&a.parent[x]);
   }
   __stcg(&a.parent[s], x);
-  int* slot = &a.broot[point_bucket<DIM>(a, a.sfeat[s])];
+  const uint32_t b = a.sbkt[s];
+  const unsigned peers = __match_any_sync(act, b);
+  const int lo = __reduce_min_sync(peers, x), hi = __reduce_max_sync(peers, x);
+  if ((peers & ((1u << (threadIdx.x & 31)) - 1u)) != 0u) return;
+  int* slot = &a.broot[b];
+  if (lo != hi) {
+    atomicExch(slot, -1);
+    return;
+  }
   const int old = atomicCAS(slot, kNoCore, x);
   if (old != kNoCore && old != x && old != -1) atomicExch(slot, -1);
 }
 
-// the smallest original core index of each component, at its root
+// the smallest original core index of each component, at its root (the lanes
+// of a warp that share a root send one)
 __global__ void k_cmin(ClusterArgs a) {
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= a.n || !a.score[s]) return;
-  atomicMin(&a.cmin[uf_find(a.parent, (int)s)], a.sidx[s]);
+  const bool core = s < a.n && a.score[s];
+  const unsigned act = __ballot_sync(kFull, core);
+  if (!core) return;
+  const int r = uf_find(a.parent, (int)s);
+  const unsigned peers = __match_any_sync(act, r);
+  const int m = __reduce_min_sync(peers, a.sidx[s]);
+  if ((peers & ((1u << (threadIdx.x & 31)) - 1u)) == 0u) atomicMin(&a.cmin[r], m);
 }
 
 // Core points: root = the component's smallest core index; border points:
@@ -490,7 +567,7 @@ __global__ void k_roots(ClusterArgs a, int* root) {
   bool alone = false;
   if (need) {
     const float4 fp = a.sfeat[s];
-    const Cell c = cell_of<DIM>(a, fp);
+    const Cell c = cell_at(a, s);
     alone = cand_count<DIM>(a, c) <= kAloneMax;
     if (alone) {  // a sparse neighbourhood: walk it alone
       int best = 0x7fffffff;
@@ -515,7 +592,7 @@ __global__ void k_roots(ClusterArgs a, int* root) {
     const int64_t sl = s - lane + l;
     const float4 fl = a.sfeat[sl];
     int best = 0x7fffffff;  // warp-uniform
-    coop_walk<DIM>(a, cell_of<DIM>(a, fl), [&](int base, int e) {
+    coop_walk<DIM>(a, cell_at(a, sl), [&](int base, int e) {
       int mine = 0x7fffffff;
 #pragma unroll
       for (int w = 0; w < kCoopW; ++w) {
@@ -775,13 +852,16 @@ cudaError_t launch_grid_phase(ClusterArgs& a, int64_t buckets, int* excl, int* b
   k_starts<<<grid_for(buckets + 1), kCT, 0, s>>>(a, excl, block_sum, buckets);
   k_scatter<DIM><<<grid_for(a.n), kCT, 0, s>>>(a);
   k_core<DIM><<<grid_for(a.n), kCT, 0, s>>>(a);
-  k_union_near<DIM><<<grid_for(a.n), kCT, 0, s>>>(a);
-  k_compress<<<grid_for(a.n), kCT, 0, s>>>(a);
+  k_link_blocks<DIM><<<(unsigned)((a.n + kLT - 1) / kLT), kLT, 0, s>>>(a);
   // the bucket counts are consumed by now: their memory holds the bucket roots
-  const cudaError_t e = cudaMemsetAsync(a.broot, 0xfe, (size_t)buckets * 4, s);
+  cudaError_t e = cudaMemsetAsync(a.broot, 0xfe, (size_t)buckets * 4, s);
   if (e != cudaSuccess) return e;
-  k_bucket_roots<DIM><<<grid_for(a.n), kCT, 0, s>>>(a);
-  k_union<DIM><<<grid_for(a.n), kCT, 0, s>>>(a);
+  k_bucket_roots<<<grid_for(a.n), kCT, 0, s>>>(a);
+  k_union<DIM, true><<<grid_for((a.n + kSample - 1) / kSample * kUGSampled), kCT, 0, s>>>(a);
+  e = cudaMemsetAsync(a.broot, 0xfe, (size_t)buckets * 4, s);
+  if (e != cudaSuccess) return e;
+  k_bucket_roots<<<grid_for(a.n), kCT, 0, s>>>(a);
+  k_union<DIM, false><<<grid_for(a.n * kUGRest), kCT, 0, s>>>(a);
   k_cmin<<<grid_for(a.n), kCT, 0, s>>>(a);
   k_roots<DIM><<<grid_for(a.n), kCT, 0, s>>>(a, root);
   return cudaSuccess;
@@ -866,6 +946,7 @@ cudaError_t launch_cluster(const float* feat, int64_t n, int dim, double eps, in
   a.bslot = bslot;
   a.sfeat = sfeat;
   a.sidx = sidx;
+  a.sbkt = (uint32_t*)keys;  // the keys are written once no kernel needs the buckets any more
   a.score = score;
   a.core = core;
   a.parent = parent;
