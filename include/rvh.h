@@ -344,9 +344,9 @@ int rvh_get_stats(rvh_ctx* ctx, rvh_stats* out);
 int rvh_set_schedule(rvh_ctx* ctx, int32_t points_per_warp, int32_t hyps_per_lane);
 
 /* Staged scoring with exact pruning (default on): the scoring pass of a
- * cluster of 256 to 32767 points (the lanes-over-trials schedule,
- * points_per_warp 1) runs in stages, the first
- * two of 128 points and each later one twice as long.  After the first,
+ * cluster of 256 (3D: 128) to 32767 points (the lanes-over-trials schedule,
+ * points_per_warp 1) runs in stages, the first of 128 (3D: 64) points, the
+ * second of 128 and each later one twice as long.  After the first,
  * the trial with the highest partial count leads: it is counted over every
  * point, and its residuals bound how many of the points still to come any
  * other trial can hold.  After each stage a trial whose partial count plus

@@ -151,28 +151,34 @@ __device__ bool hyp_f64(const FrameDesc& a, const RS& R, int ci, int h, int N, d
 //   - points with |r_L| <= tau + max|a.d|, of those the lead does not hold, and
 //   - points with |a.d| <= tau + |r_L| <= 2 tau, of those it does: with
 //     t = a1 / a0 (the tangent of the azimuth) that is an interval of t,
-//     |d0 + d1 t| <= (2 tau + max|a2 d2|) / min a0.
-// Two histograms over the points still to be scored -- the excess |r_L| -
+//     |d0 + d1 t + a2 d2 / a0| <= 2 tau / a0.  In 3D a2 d2 varies with the
+//     elevation, and d2 is large (elevations span little, so trials differ
+//     most in their vertical velocity): the lower and the upper half of a2's
+//     range have an interval each.
+// Histograms over the points still to be scored -- the excess |r_L| -
 // thi of the points outside the lead, a quarter octave per bin, and t of the
-// points inside, evenly over the cluster's range -- turn both into counts
+// points inside, evenly over the cluster's range, per half of a2 -- turn both into counts
 // per trial, which replace "every point still to come" in the pruning test.
 // Everything is rounded so that the counts only err upwards: bins are taken
 // by the same monotone FP32 expressions on both sides, and the band
 // half-widths of both trials (which bound the FP32 residuals' and
 // velocities' errors) are added to the thresholds.
 constexpr int kExcessBins = 64, kTanBins = 32;
+template <int DIM>
+constexpr int kHalves = DIM == 3 ? 2 : 1;
 constexpr int kExcessBase = 119 << 2;  // bin 0: an excess below 2^-8 m/s
 
 __device__ __forceinline__ int excess_bin(float x) {
   return min(max((__float_as_int(x) >> 21) - kExcessBase, 0), kExcessBins - 1);
 }
 
-// The cluster's directions a: range of t = a1 / a0, 1 / min a0 and max|a2|;
+// The cluster's directions a: range of t = a1 / a0, 1 / min a0, max|a2|, and
+// the least a2 and a quarter of its range (a half's centre and half-width);
 // tan_ok = 0 (some a0 not safely positive) leaves the interval test out.
 // The line model's rows (x, 1, y) have residuals of the same form with a =
 // (1, x): t = x in [0, 1], a0 = 1, and the components of d change places.
 struct DirRange {
-  float t0, tinv, tabs, a0inv, zmax;
+  float t0, tinv, tabs, a0inv, zmax, z0, zq;
   int tan_ok;
 };
 
@@ -211,12 +217,13 @@ __device__ __forceinline__ float record_tlo(float4 hy, TauPair tau, bool line) {
 }
 
 // Where a trial's points can lie, as bins: excess bins 0 .. out of the points
-// outside the lead, t bins lo .. hi - 1 of those inside.  Packed in one word.
+// outside the lead, t bins lo .. hi - 1 of those inside, per half of a2.
+// Packed in one word, six bits each.
 struct HoldRange {
   uint32_t v;
-  __device__ __forceinline__ int out() const { return (int)(v & 255u); }
-  __device__ __forceinline__ int lo() const { return (int)(v >> 8 & 255u); }
-  __device__ __forceinline__ int hi() const { return (int)(v >> 16); }
+  __device__ __forceinline__ int out() const { return (int)(v & 63u); }
+  __device__ __forceinline__ int lo(int c) const { return (int)(v >> (6 + 12 * c) & 63u); }
+  __device__ __forceinline__ int hi(int c) const { return (int)(v >> (12 + 12 * c) & 63u); }
 };
 
 template <int DIM>
@@ -229,16 +236,33 @@ __device__ __forceinline__ HoldRange hold_range(const DirRange& g, float4 lead, 
   const float slack = 2.0f * lead_band + 4e-6f * (ax + ay + fabsf(dz));
   // max|a.d|: unit directions, or the ends of x's range for the line model
   const float reach = line ? fmaxf(ax, fabsf(dx + dy)) : sqrt_approx(fmaf(dx, dx, dy * dy)) + az;
-  const uint32_t out = (uint32_t)excess_bin((hy.w + reach + slack) * 1.0001f - lead.w);
-  uint32_t lo = 0u, hi = kTanBins;
-  if (g.tan_ok) {
-    const float K = (hy.w + lead.w + slack + az) * g.a0inv * 1.0001f + 1e-5f * (ax + ay * g.tabs);
-    const float r = rcp_approx(dy);  // dy = 0: ends at +-inf, all of t or none of it
-    const float u = (-dx - K) * r, v = (K - dx) * r;
-    lo = (uint32_t)min(max(__float2int_rd((fminf(u, v) - g.t0) * g.tinv), 0), kTanBins);
-    hi = (uint32_t)max(min(__float2int_rd((fmaxf(u, v) - g.t0) * g.tinv), kTanBins - 1) + 1, (int)lo);
+  HoldRange h;
+  h.v = (uint32_t)excess_bin((hy.w + reach + slack) * 1.0001f - lead.w);
+  const float r = rcp_approx(dy);  // dy = 0: ends at +-inf, all of t or none of it
+#pragma unroll
+  for (int c = 0; c < kHalves<DIM>; ++c) {
+    uint32_t lo = 0u, hi = kTanBins;
+    if (g.tan_ok) {
+      float u, v;
+      if (DIM == 2) {
+        const float K = (hy.w + lead.w + slack) * g.a0inv * 1.0001f + 1e-5f * (ax + ay * g.tabs);
+        u = (-dx - K) * r;
+        v = (K - dx) * r;
+      } else {
+        // a0 (d0 + d1 t) within K0 of -a2 dz, a0 in [min a0, 1]
+        const float mid = (g.z0 + (float)(2 * c + 1) * g.zq) * dz;
+        const float K0 = (hy.w + lead.w + slack + g.zq * fabsf(dz)) * 1.0001f;
+        const float s = 1e-5f * (ax + ay * g.tabs + az + K0);
+        const float A = -K0 - mid - s, B = K0 - mid + s;
+        u = ((A < 0.0f ? A * g.a0inv * 1.0001f : A) - s - dx) * r;
+        v = ((B > 0.0f ? B * g.a0inv * 1.0001f : B) + s - dx) * r;
+      }
+      lo = (uint32_t)min(max(__float2int_rd((fminf(u, v) - g.t0) * g.tinv), 0), kTanBins);
+      hi = (uint32_t)max(min(__float2int_rd((fmaxf(u, v) - g.t0) * g.tinv), kTanBins - 1) + 1, (int)lo);
+    }
+    h.v |= lo << (6 + 12 * c) | hi << (12 + 12 * c);
   }
-  return HoldRange{out | lo << 8 | hi << 16};
+  return h;
 }
 
 struct ClusterShared {
@@ -269,12 +293,12 @@ struct ClusterShared {
   unsigned long long scored;   // (trial, point) pairs the scoring pass evaluated
   int nref;                   // 2D trials queued for refinement in the current chunk
   DirRange dir;               // the cluster's directions (staged pass)
-  int red_d[4][kWarps];
+  int red_d[5][kWarps];
   // Points still to be scored when the lead was taken, by its residual:
-  // inside it, those below each bin of t; outside it, those up to each bin of
-  // the excess.  From stage 0 / 1 on and, in the second half, from 2 / 3 on,
-  // as 16-bit halves.
-  unsigned lead_in[2 * (kTanBins + 1)];
+  // inside it, those below each bin of t per half of a2; outside it, those up
+  // to each bin of the excess.  From stage 0 / 1 on and, in the second half of
+  // the array, from 2 / 3 on, as 16-bit halves.
+  unsigned lead_in[2 * 2 * (kTanBins + 1)];
   unsigned lead_out[2 * kExcessBins];
   unsigned lead_cnt;          // the lead's certain points and band points
 };
@@ -1010,12 +1034,18 @@ __device__ __forceinline__ int prune_list(const Smem& S, int n, Keep keep, int* 
 // frame (dense2d / stress2d / dense3d): without the pass 0.292 / 0.846 /
 // 1.93; pruning by "every point still to come" instead of the lead's
 // residuals (72% / 100% / 66% of the pairs) 0.261 / 0.845 / 1.688; this pass
-// (42% / 59% / 38%) 0.221 / 0.787 / 1.480.  First stage of 64 / 96 / 128
+// (42% / 59% / 38%) 0.221 / 0.787 / 1.480.  2D: first stage of 64 / 96 / 128
 // points 0.229 / 0.224 / 0.221 (a longer one finds a better lead), threshold
-// of 192 instead of 256 points 0.223 / 0.802 / 1.495; a new lead after every
-// early stage evaluates fewer pairs (29%) but took 0.305 ms.
-constexpr int kStage0Quads = 32, kStage1Quads = 32;
-constexpr int kStageMinPoints = 256;
+// of 192 instead of 256 points 0.223 / 0.802; a new lead after every early
+// stage evaluates fewer pairs (29%) but took 0.305 ms.  3D with an interval
+// per half of a2 (27% of the pairs): 1.372 -> 1.229 ms, and with its tighter
+// first test a first stage of 96 / 64 points 1.218 / 1.220, threshold 192 /
+// 128 points at 64 1.210 / 1.209.
+template <int DIM>
+constexpr int kStage0Quads = DIM == 2 ? 32 : 16;
+constexpr int kStage1Quads = 32;
+template <int DIM>
+constexpr int kStageMinPoints = DIM == 2 ? 256 : 128;
 constexpr int kStageMaxPoints = 32767;  // points are counted in 16-bit halves
 
 // The cluster's direction range (DirRange) from this thread's own rows: each
@@ -1025,35 +1055,41 @@ template <int DIM, typename RV>
 __device__ __forceinline__ void direction_range(const RV rows, int N, bool line, ClusterShared& cs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float inf = __int_as_float(0x7f800000);
-  float a0 = inf, t0 = inf, t1 = -inf, z = 0.0f;
+  float a0 = inf, t0 = inf, t1 = -inf, z0 = inf, z1 = -inf;
   for (int j = tid; j < N; j += kThreads) {
     const float4 p = rows.at(j);
     const float t = row_tan(p, line);
     a0 = fminf(a0, line ? p.y : p.x);
     t0 = fminf(t0, t);
     t1 = fmaxf(t1, t);
-    if (DIM == 3) z = fmaxf(z, fabsf(p.z));
+    if (DIM == 3) {
+      z0 = fminf(z0, p.z);
+      z1 = fmaxf(z1, p.z);
+    }
   }
   const int r0 = __reduce_min_sync(0xffffffffu, float_order(a0)), r1 = __reduce_min_sync(0xffffffffu, float_order(t0)),
             r2 = __reduce_max_sync(0xffffffffu, float_order(t1)),
-            r3 = DIM == 3 ? __reduce_max_sync(0xffffffffu, float_order(z)) : 0;
+            r3 = DIM == 3 ? __reduce_min_sync(0xffffffffu, float_order(z0)) : 0,
+            r4 = DIM == 3 ? __reduce_max_sync(0xffffffffu, float_order(z1)) : 0;
   if (lane == 0) {
     cs.red_d[0][warp] = r0;
     cs.red_d[1][warp] = r1;
     cs.red_d[2][warp] = r2;
     cs.red_d[3][warp] = r3;
+    cs.red_d[4][warp] = r4;
   }
 }
 
 template <int DIM>
 __device__ __forceinline__ void direction_range_finish(ClusterShared& cs) {
   if (threadIdx.x != 0) return;
-  int r[4];
+  int r[5];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < (DIM == 3 ? 5 : 3); ++i) {
     r[i] = cs.red_d[i][0];
 #pragma unroll
-    for (int w = 1; w < kWarps; ++w) r[i] = i < 2 ? min(r[i], cs.red_d[i][w]) : max(r[i], cs.red_d[i][w]);
+    for (int w = 1; w < kWarps; ++w)
+      r[i] = i == 2 || i == 4 ? max(r[i], cs.red_d[i][w]) : min(r[i], cs.red_d[i][w]);
   }
   const float a0 = order_float(r[0]), t0 = order_float(r[1]), t1 = order_float(r[2]);
   const float inv = __fdividef(kTanBins - 0.01f, t1 - t0);
@@ -1061,8 +1097,16 @@ __device__ __forceinline__ void direction_range_finish(ClusterShared& cs) {
   cs.dir.tinv = t1 > t0 && inv < 1e30f ? inv : 0.0f;  // else one bin holds them all
   cs.dir.tabs = fmaxf(fabsf(t0), fabsf(t1));
   cs.dir.a0inv = rcp_approx(a0) * kRcpUp;
-  cs.dir.zmax = DIM == 3 ? order_float(r[3]) : 0.0f;
   cs.dir.tan_ok = a0 > 1e-3f && a0 < 2.0f;
+  if (DIM == 3) {
+    const float z0 = order_float(r[3]), z1 = order_float(r[4]);
+    cs.dir.zmax = fmaxf(fabsf(z0), fabsf(z1));
+    cs.dir.z0 = z0;
+    // a little wide: centre +- zq holds its half whatever the rounding
+    cs.dir.zq = 0.25f * (z1 - z0) + 1e-6f;
+  } else {
+    cs.dir.zmax = cs.dir.z0 = cs.dir.zq = 0.0f;
+  }
 }
 
 // Scores the chunk's normal trials in stages.  After the first stage the
@@ -1096,13 +1140,14 @@ __device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, co
       u += a1 - a0;
     }
   };
-  if (tid < 2 * (kTanBins + 1)) cs.lead_in[tid] = 0u;
+  constexpr int NH = kHalves<DIM>, kIn = NH * (kTanBins + 1);
+  if (tid < 2 * kIn) cs.lead_in[tid] = 0u;
   if (tid < 2 * kExcessBins) cs.lead_out[tid] = 0u;
   unsigned long long lim = cs.best;  // the key to beat
   int q0 = 0, lead = -1;
   float4 lw = cs.win;
   if (lim == 0ull || !(lw.w < 1e30f)) {  // no lead with an FP32 record yet
-    score(std::false_type{}, nh, 0, kStage0Quads);
+    score(std::false_type{}, nh, 0, kStage0Quads<DIM>);
     top = __reduce_max_sync(0xffffffffu, top);
     if (lane == 0) cs.red_i[warp] = (int)top;
     __syncthreads();
@@ -1110,7 +1155,7 @@ __device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, co
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) top = max(top, (unsigned)cs.red_i[w]);
     if (top == 0u) return scored;  // no normal trial
-    q0 = kStage0Quads;
+    q0 = kStage0Quads<DIM>;
     lead = 0xFFFF - (int)(top & 0xFFFFu);
     lw = S.hyp[lead];
   } else {
@@ -1131,7 +1176,10 @@ __device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, co
       if (q >= q0) {
         const unsigned one = (q < e1 || (q >= e2 && q < e3)) ? 1u : 1u << 16;
         if (r <= lw.w)
-          atomicAdd(&cs.lead_in[(q < e2 ? 0 : kTanBins + 1) + tan_bin(dir, row_tan(p, line))], one);
+          atomicAdd(&cs.lead_in[(q < e2 ? 0 : kIn) +
+                                (DIM == 3 && p.z >= dir.z0 + 2.0f * dir.zq ? kTanBins + 1 : 0) +
+                                tan_bin(dir, row_tan(p, line))],
+                    one);
         else if (r > lw.w)  // NaN: held by no trial
           atomicAdd(&cs.lead_out[(q < e2 ? 0 : kExcessBins) + excess_bin(r - lw.w)], one);
       }
@@ -1139,10 +1187,10 @@ __device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, co
     cnt = __reduce_add_sync(0xffffffffu, cnt);
     if (lane == 0) cs.red_i[warp] = (int)cnt;
     __syncthreads();
-    if (warp < 2) {
-      unsigned* h = warp == 0 ? cs.lead_in : cs.lead_out;
-      const int stride = warp == 0 ? kTanBins + 1 : kExcessBins;
-      const int b = warp == 0 ? lane : 2 * lane;
+    if (warp < 1 + NH) {  // warp 1: outside, the others: inside, a half of a2 each
+      unsigned* h = warp == 1 ? cs.lead_out : cs.lead_in + (warp >> 1) * (kTanBins + 1);
+      const int stride = warp == 1 ? kExcessBins : kIn;
+      const int b = warp == 1 ? 2 * lane : lane;
       uint2 c0 = make_uint2(h[b], h[stride + b]), c1 = make_uint2(0u, 0u);
       if (warp == 1) c1 = make_uint2(h[b + 1], h[stride + b + 1]);
       uint2 incl = make_uint2(c0.x + c1.x, c0.y + c1.y);
@@ -1161,14 +1209,14 @@ __device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, co
         h[bin] = x;
         h[stride + bin] = y;
       };
-      if (warp == 0) {
-        put(lane, incl.x - c0.x, incl.y - c0.y);
-        if (lane == 31) put(kTanBins, incl.x, incl.y);
-      } else {
+      if (warp == 1) {
         put(b, incl.x - c1.x, incl.y - c1.y);
         put(b + 1, incl.x, incl.y);
+      } else {
+        put(lane, incl.x - c0.x, incl.y - c0.y);
+        if (lane == 31) put(kTanBins, incl.x, incl.y);
       }
-    } else if (warp == 2) {
+    } else if (warp == 3) {
       const unsigned v = __reduce_add_sync(0xffffffffu, lane < kWarps ? (unsigned)cs.red_i[lane] : 0u);
       if (lane == 0) cs.lead_cnt = v;
     }
@@ -1196,10 +1244,12 @@ __device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, co
   // the pruning test before stage s: the points from it on that trial h can hold
   auto keep = [&](int h, HoldRange r, int s) {
     const int sh = (s & 1) << 4;
-    const unsigned* in = cs.lead_in + (s >> 1) * (kTanBins + 1);
-    const unsigned* out = cs.lead_out + (s >> 1) * kExcessBins;
-    const int n = (int)(out[r.out()] >> sh & 0xFFFFu) + (int)(in[r.hi()] >> sh & 0xFFFFu) -
-                  (int)(in[r.lo()] >> sh & 0xFFFFu);
+    const unsigned* in = cs.lead_in + (s >> 1) * kIn;
+    int n = (int)(cs.lead_out[(s >> 1) * kExcessBins + r.out()] >> sh & 0xFFFFu);
+#pragma unroll
+    for (int c = 0; c < NH; ++c)
+      n += (int)(in[c * (kTanBins + 1) + r.hi(c)] >> sh & 0xFFFFu) -
+           (int)(in[c * (kTanBins + 1) + r.lo(c)] >> sh & 0xFFFFu);
     const bool k = best_key(S.U[h] + n, hc0 + h) > lim;
     if (!k) S.U[h] = -1;
     return k;
@@ -1399,7 +1449,7 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
     cs.best = 0ull;
     cs.nref = 0;
   }
-  const bool may_stage = prune && pw == 1 && N >= kStageMinPoints && N <= kStageMaxPoints;
+  const bool may_stage = prune && pw == 1 && N >= kStageMinPoints<DIM> && N <= kStageMaxPoints;
   const bool line = EXT && DIM == 2 && a.line_model;
   if (may_stage) direction_range<DIM>(rows, N, line, cs);
   const float wmax = block_max_float(wm, cs.red_f);  // its barrier also orders the row writes

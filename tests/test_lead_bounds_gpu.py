@@ -30,6 +30,8 @@ def _cluster(kind, n, dim, rng):
         az = rng.uniform(-3.1, 3.1, n)
     elif kind == "narrow":  # a far object: every direction nearly alike
         az = 0.7 + rng.uniform(-2e-3, 2e-3, n)
+    elif kind == "flat":  # one elevation: both halves of its range are one value
+        el = np.full(n, 0.1)
     elif kind == "two":  # two directions only: histogram range of two values
         az = np.where(rng.random(n) < 0.5, -0.4, 0.4)
     if dim == 2:
@@ -52,9 +54,9 @@ def _cluster(kind, n, dim, rng):
 def test_bounds_keep_every_result(ctx, dim, H):
     from paper_2012_12618_gb300 import rvh
     rng = np.random.default_rng(dim * 7 + H)
-    # around the staging threshold, the stage ends (128, 256, 512, 1024 points) and the row capacity
-    sizes = [255, 256, 257, 300, 511, 513, 639, 1023, 1025, 1536, 1537, 2047, 2048]
-    parts = [_cluster(k, n, dim, rng) for k in ("wide", "behind", "narrow", "two", "same", "step") for n in sizes]
+    # around the staging thresholds (3D 128, 2D 256), the stage ends and the row capacity
+    sizes = [127, 128, 129, 191, 193, 255, 256, 257, 300, 511, 513, 639, 1023, 1025, 1536, 1537, 2047, 2048]
+    parts = [_cluster(k, n, dim, rng) for k in ("wide", "behind", "narrow", "flat", "two", "same", "step") for n in sizes]
     az, el, dop = (np.concatenate([p[i] for p in parts]) for i in range(3))
     off = np.concatenate([[0], np.cumsum([len(p[0]) for p in parts])]).astype(np.int32)
     kw = dict(el=el if dim == 3 else None, H=H, tau=0.1, seed=5)
