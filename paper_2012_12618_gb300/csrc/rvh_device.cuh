@@ -93,6 +93,23 @@ __device__ __forceinline__ void sincos_f64(const double2* __restrict__ trig, flo
   *s = fma(cs.y, cm1, fma(cs.x, sx, cs.y));
 }
 
+// atan2(y, x) from the row table: the FP32 angle picks the nearest k/128,
+// tan(theta - k/128) = (y cos - x sin) / (x cos + y sin) of that table entry is
+// below 2^-8 + 2^-20, and arctangent's Taylor series to the seventh power gives
+// the rest (the ninth is below 2^-75).  Within 3 x 2^-52 of the angle (1.5
+// units in its last place at pi), with about half the FP64 chain of the
+// library's atan2.  Arguments outside 1e-30 .. 1e30 go to the library.
+__device__ __forceinline__ double atan2_table(const double2* __restrict__ trig, double y, double x) {
+  const double m = fmax(fabs(x), fabs(y));
+  if (!(m >= 1e-30 && m <= 1e30)) return atan2(y, x);
+  const float k = rintf(atan2f((float)y, (float)x) * 128.0f);
+  const double2 cs = __ldg(&trig[(int)k + kTrigHalf]);
+  const double d = fma(y, cs.x, -(x * cs.y)) / fma(x, cs.x, y * cs.y);
+  const double d2 = d * d;
+  const double p = fma(d2, fma(d2, -1.0 / 7.0, 1.0 / 5.0), -1.0 / 3.0);
+  return (double)(k * 0.0078125f) + fma(d * d2, p, d);
+}
+
 // Rows of A_i (Eq. eq:LSQPerCluster) in FP64: (cos t, sin t) or
 // (cos t cos e, sin t cos e, sin e).
 template <int DIM>

@@ -758,9 +758,8 @@ __device__ __forceinline__ bool solve_normal(const double* t, int n_in, double v
   }
 }
 
-// Final solve and heading of a cluster: the normal equations, with a
-// fallback to the winning minimal-set velocity, heading atan2(vy, vx).
-// One thread.
+// Final solve of a cluster: the normal equations, with a fallback to the
+// winning minimal-set velocity (whose heading is formed here too).  One thread.
 template <int DIM, bool EXT>
 __device__ __noinline__ void finish_cluster(const FrameDesc& a, const Rows64Inputs<DIM>& R, int ci, int N, int hstar, int n_in,
                                const double* t, const double* v64, bool has_v64) {
@@ -778,17 +777,46 @@ __device__ __noinline__ void finish_cluster(const FrameDesc& a, const Rows64Inpu
     } else {
       if (!has_v64) hyp_f64<DIM>(a, R, ci, hstar, N, vout);
     }
+    a.heading[ci] = atan2(vout[1], vout[0]);
   }
   a.vx[ci] = vout[0];
   a.vy[ci] = vout[1];
   if (a.vz) a.vz[ci] = DIM == 3 ? vout[2] : 0.0;
-  a.heading[ci] = atan2(vout[1], vout[0]);
   a.inlier_count[ci] = n_in;
   a.best[ci] = hstar;
   a.status[ci] = st;
 }
 
-// A cluster waiting for its final solve and heading (finish_cluster): the
+// Heading of a cluster whose normal equations are solvable (else
+// finish_cluster forms it): atan2 of Cramer's numerators, so that it does not
+// wait for the velocity's divisions.  One thread, in another warp than
+// finish_cluster's.  A frame of few clusters ends with these two, one cluster
+// per CTA: one thread doing both, with the library's atan2, took 2.8 us of it;
+// 64 clusters 20.6 -> 19.5 us.
+template <int DIM>
+__device__ __noinline__ void finish_heading(const FrameDesc& a, int ci, int n_in, const double* t) {
+  if (!normal_solvable<DIM>(t, n_in)) return;
+  double det, x, y;
+  if (DIM == 2) {
+    det = det2_f64(t[0], t[1], t[1], t[2]);
+    x = det2_f64(t[3], t[1], t[4], t[2]);
+    y = det2_f64(t[0], t[3], t[1], t[4]);
+  } else {
+    const double G0[3] = {t[0], t[1], t[2]}, G1[3] = {t[1], t[3], t[4]}, G2[3] = {t[2], t[4], t[5]};
+    const double A0[3] = {t[6], t[1], t[2]}, A1[3] = {t[7], t[3], t[4]}, A2[3] = {t[8], t[4], t[5]};
+    const double B0[3] = {t[0], t[6], t[2]}, B1[3] = {t[1], t[7], t[4]}, B2[3] = {t[2], t[8], t[5]};
+    det = det3_f64(G0, G1, G2);
+    x = det3_f64(A0, A1, A2);
+    y = det3_f64(B0, B1, B2);
+  }
+  if (det < 0.0) {
+    x = -x;
+    y = -y;
+  }
+  a.heading[ci] = atan2_table(a.trig, y, x);
+}
+
+// A cluster waiting for its final solve and heading: the
 // CTA queues up to kFinishBatch of them in shared memory and finishes them
 // together, one lane each.  Serial FP64 on one lane costs as much pipe time
 // per instruction as a full warp, so a lone thread finishing each cluster
@@ -1654,16 +1682,21 @@ __global__ void __launch_bounds__(kThreads, RVH_MIN_BLOCKS) fused_kernel(const _
     fq_n = 0;
     cs.scored = 0ull;
   }
-  // the queued clusters' solves and headings, one lane each
+  // the queued clusters' solves (warp 0) and headings (warp 1), one lane each
   auto flush = [&]() {
     const int n = fq_n;
-    if (threadIdx.x < n) {
-      const FinishRec& q = fq[threadIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < 2 && lane < n) {
+      const FinishRec& q = fq[lane];
       const FrameDesc& F = a.f[q.frame];
-      // the CTA's row slot has moved on to later clusters: rows are
-      // recomputed for the (rare) fallback solve
-      const Rows64Inputs<DIM> R = {&F, q.o};
-      finish_cluster<DIM, EXT>(F, R, q.ci, q.N, q.hstar, q.n_in, q.t, q.v64, q.has_v64 != 0);
+      if (warp == 0) {
+        // the CTA's row slot has moved on to later clusters: rows are
+        // recomputed for the (rare) fallback solve
+        const Rows64Inputs<DIM> R = {&F, q.o};
+        finish_cluster<DIM, EXT>(F, R, q.ci, q.N, q.hstar, q.n_in, q.t, q.v64, q.has_v64 != 0);
+      } else {
+        finish_heading<DIM>(F, q.ci, q.n_in, q.t);
+      }
     }
     __syncthreads();
     if (threadIdx.x == 0) fq_n = 0;
