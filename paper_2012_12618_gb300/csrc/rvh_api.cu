@@ -56,6 +56,9 @@ int fail(int code, const std::string& msg) {
   } while (0)
 
 constexpr size_t kAlign = 256;
+// One copy of the launch counters: the two that graph launches take in turn,
+// then the one of plain launches (a captured call may run again at any time).
+constexpr size_t kStatsBytes = 128;
 size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 
 bool is_device_ptr(const void* p) {
@@ -179,6 +182,7 @@ struct rvh_ctx {
   cudaEvent_t last_done = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   unsigned long long* stats_d = nullptr;
+  int stats_slot = 0;  // the counters' clean copy (launch_graph): used by the next call, which cleans the other
   bool have_launch = false;
   rvh_stats last{};
   int pw_fixed = 0, hpl_fixed = 0;
@@ -336,22 +340,23 @@ int launch_batch(rvh_ctx* ctx, FusedArgs& a, int dim, cudaStream_t s, cudaEvent_
 
 // Launches the fused kernel through the context's CUDA graph of its kernel
 // instantiation, the call's arguments written into the graph's kernel node
-// (rvh_graph.cu).  The stats reset, the work-list kernel and the timing
-// events stay outside the graph, so the events time the fused kernel.
+// (rvh_graph.cu).  The work-list kernel and the timing
+// events stay outside the graph, so the events time the fused kernel.  The
+// counters have two copies: each launch adds to the clean one and zeroes the
+// other for the next (a memset before each launch took 2 us of a small frame).
 int launch_graph(rvh_ctx* ctx, FusedArgs& a, int dim, cudaStream_t s) {
   int grid = 1;
   size_t smem = 0;
   int rc = prepare_launch(ctx, a, dim, &grid, &smem);
   if (rc) return rc;
-  // the work-list kernel zeroes the stats; a direct launch has none before it
-  if (a.direct) RVH_CUDA(cudaMemsetAsync(a.stats, 0, sizeof(unsigned long long) * kStatsWords, s));
-  else RVH_CUDA(launch_worklist(a, s));
+  if (!a.direct) RVH_CUDA(launch_worklist(a, s));
   RVH_CUDA(cudaEventRecord(ctx->ev0, s));
   const cudaError_t e = ctx->graph[dim == 3][fused_ext(a) ? 1 : 0].launch(a, dim, grid, smem, false, s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(RVH_ECUDA, std::string("graph launch: ") + cudaGetErrorString(e));
   }
+  ctx->stats_slot ^= 1;
   RVH_CUDA(cudaEventRecord(ctx->ev1, s));
   ctx->last.grid = grid;
   ctx->last.kernel_launches = a.direct ? 1 : 2;
@@ -645,9 +650,9 @@ static int stage(rvh_ctx* ctx, const rvh_frame* f, const rvh_params* p, rvh_resu
     off += align_up(bytes);
     return o;
   };
+  const size_t o_stats = take(3 * kStatsBytes);  // first: its place does not depend on the frame
   const size_t o_work = take(sizeof(int2) * (size_t)std::max(nc, 1));
   const size_t o_ctr = take(64);
-  const size_t o_stats = take(128);
   const size_t o_rows = take((fused ? sizeof(float4) : 4 * sizeof(double)) * (size_t)std::max<int64_t>(np, 1));
   const size_t o_rows64 = fused ? take(sizeof(double4_32a) * (size_t)std::max<int64_t>(np, 1)) : 0;
   size_t o_cta64 = 0;
@@ -677,6 +682,7 @@ static int stage(rvh_ctx* ctx, const rvh_frame* f, const rvh_params* p, rvh_resu
     int rc = ctx_alloc(ctx, &ctx->scratch, want);
     if (rc) return rc;
     ctx->scratch_bytes = want;
+    RVH_CUDA(cudaMemsetAsync(ctx->scratch, 0, 3 * kStatsBytes, s));
   }
   char* b = (char*)ctx->scratch;
   st.base = b;
@@ -731,7 +737,6 @@ int rvh_estimate(rvh_ctx* ctx, const rvh_frame* frame, const rvh_params* params,
   Staged st{};
   rc = stage(ctx, frame, params, result, s, true, st);
   if (rc) return rc;
-  ctx->stats_d = st.stats;
   FusedArgs a;
   memset(&a, 0, sizeof(a));
   fill_desc(ctx->trig, a.f[0], *frame, *params, st.az, st.el, st.dop, st.off, (float4*)st.rows, st.rows64,
@@ -740,15 +745,19 @@ int rvh_estimate(rvh_ctx* ctx, const rvh_frame* frame, const rvh_params* params,
   a.n_items = frame->n_clusters;
   a.worklist = st.worklist;
   a.work_counter = st.counter;
-  a.stats = st.stats;
   a.cta_rows64 = ctx->cta_rows ? st.cta_rows64 : nullptr;
   choose_schedule(ctx, params->model_dim, trials_per_chunk(*params), &a.pw, &a.hpl);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   RVH_CUDA(cudaStreamIsCapturing(s, &cap));
+  constexpr size_t kStride = kStatsBytes / sizeof(unsigned long long);
   if (ctx->graphs && s != nullptr && cap == cudaStreamCaptureStatusNone) {
+    a.stats = st.stats + (size_t)ctx->stats_slot * kStride;
+    a.stats_next = st.stats + (size_t)(ctx->stats_slot ^ 1) * kStride;
+    ctx->stats_d = a.stats;
     rc = launch_graph(ctx, a, params->model_dim, s);
   } else {
-    RVH_CUDA(cudaMemsetAsync(st.stats, 0, sizeof(unsigned long long) * kStatsWords, s));
+    a.stats = ctx->stats_d = st.stats + 2 * kStride;
+    RVH_CUDA(cudaMemsetAsync(a.stats, 0, sizeof(unsigned long long) * kStatsWords, s));
     rc = launch_batch(ctx, a, params->model_dim, s, ctx->ev0, ctx->ev1);
   }
   if (rc) return rc;

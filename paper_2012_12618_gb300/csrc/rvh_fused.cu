@@ -1673,6 +1673,7 @@ __global__ void __launch_bounds__(kThreads, RVH_MIN_BLOCKS) fused_kernel(const _
   p += ((size_t)a.hchunk * sizeof(int8_t) + 15) & ~(size_t)15;
   S.list = reinterpret_cast<uint16_t*>(p);
 
+  if (blockIdx.x == 0 && a.stats_next && threadIdx.x < kStatsWords) a.stats_next[threadIdx.x] = 0ull;
   if (threadIdx.x < 4) cs.ctr[threadIdx.x] = 0ull;
   if constexpr (EXT) {
     if (threadIdx.x < 2) cs.runs[threadIdx.x] = 0ull;
@@ -1779,13 +1780,11 @@ __device__ __forceinline__ int item_bucket(const FrameDesc& F, int ci) {
 }
 
 // Items are numbered frame-major; each thread keeps the buckets of its first
-// kItemsKept items in registers between the two passes.  Also zeroes the
-// launch's stats counters (the fused kernel adds to them).
+// kItemsKept items in registers between the two passes.
 constexpr int kItemsKept = 8;
 __global__ void worklist_kernel(const __grid_constant__ FusedArgs a) {
   __shared__ int hist[kCostBuckets];
   for (int b = threadIdx.x; b < kCostBuckets; b += blockDim.x) hist[b] = 0;
-  if (a.stats && threadIdx.x < kStatsWords) a.stats[threadIdx.x] = 0ull;
   __syncthreads();
   int kept[kItemsKept];
   {

@@ -63,6 +63,7 @@ struct FusedArgs {
   unsigned long long* stats;  // [kStatsWords]: exact counts, band points, fp64 trials, refined trials,
                               // 6 stage cycles, trials run, pairs of the trials run (extensions),
                               // pairs the scoring pass evaluated
+  unsigned long long* stats_next;  // [kStatsWords] zeroed by this launch for the next one (or NULL)
   int nmax_smem;
   int hchunk;
   int pw, hpl;
