@@ -179,6 +179,7 @@ struct rvh_ctx {
   size_t scratch_bytes = 0;
   void* cl_scratch = nullptr;  // scratch of rvh_cluster
   size_t cl_scratch_bytes = 0;
+  int* cl_readback = nullptr;  // page-locked, 4 ints
   cudaEvent_t last_done = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   unsigned long long* stats_d = nullptr;
@@ -474,6 +475,7 @@ void rvh_destroy(rvh_ctx* ctx) {
     for (auto& g : row) g.reset();
   if (ctx->scratch) ctx_free(ctx, ctx->scratch, ctx->scratch_bytes);
   if (ctx->cl_scratch) ctx_free(ctx, ctx->cl_scratch, ctx->cl_scratch_bytes);
+  if (ctx->cl_readback) cudaFreeHost(ctx->cl_readback);
   if (ctx->trig) ctx_free(ctx, ctx->trig, sizeof(double2) * kTrigSize);
   cudaEventDestroy(ctx->last_done);
   cudaEventDestroy(ctx->ev0);
@@ -513,9 +515,10 @@ int rvh_cluster(rvh_ctx* ctx, const float* features, int64_t n_points, int32_t d
     if (rc) return rc;
     ctx->cl_scratch_bytes = need;
   }
+  if (!ctx->cl_readback) RVH_CUDA(cudaHostAlloc((void**)&ctx->cl_readback, 4 * sizeof(int), cudaHostAllocDefault));
   int nc = 0, err = 0;
   RVH_CUDA(launch_cluster(features, n_points, dim, eps, min_pts, ctx->cl_scratch, labels, perm, offsets,
-                          max_clusters, &nc, &err, s));
+                          max_clusters, &nc, &err, ctx->cl_readback, s));
   RVH_CUDA(cudaEventRecord(ctx->last_done, s));
   *n_clusters = nc;
   if (err) return fail(RVH_ECUDA, "rvh_cluster: a union did not settle within its retry limit");

@@ -46,7 +46,15 @@ namespace {
 
 constexpr int kCT = 256;                       // threads per block of the clustering kernels
 constexpr int kUnionRetries = 1 << 20;         // cap on one union's compare-and-swap retries
-constexpr int kSumsPerThread = 64;             // block sums per thread of the one-block scan
+// Values per thread of the device-wide scan.  On 10^5 points the scans are
+// bound by launches and dependent steps, not bytes: tiles of 2048 leave 256 tile
+// sums, which the next kernel's blocks add up themselves (k_starts) or one block
+// scans with 8 a thread.  With the offsets of up to 4096 clusters from one block, a
+// memset in place of four and the counts read back into page-locked memory:
+// 106 k-point scene 484 us per pass (tiles of 256, 64 sums a thread: 509).
+constexpr int kScanPer = 8;
+constexpr int kScanTile = kCT * kScanPer;
+constexpr int kSumsPerThread = 8;              // tile sums per thread of the one-block scan
 constexpr int kBT = 1024;                      // threads of the shared-memory bitonic kernels
 constexpr int kBE = 2 * kBT;                   // keys per block of those kernels
 
@@ -62,6 +70,7 @@ struct ClusterArgs {
   int* count;          // [buckets] points per bucket
   int* start;          // [buckets + 1] first sorted position of each bucket
   int2* bslot;         // [n] (bucket, slot within the bucket) of each point
+  int2* tally;         // [n] the same memory after k_scatter: cluster counts, then placement cursors (zeroed)
   float4* sfeat;       // [n] features in sorted order, zero-padded to four
   int* sidx;           // [n] original index of each sorted position
   uint32_t* sbkt;      // [n] bucket of each sorted position
@@ -228,16 +237,31 @@ __global__ void k_grid(ClusterArgs a) {
   a.bslot[i] = make_int2((int)b, atomicAdd(&a.count[b], 1));
 }
 
-// start[b] = exclusive scan of the counts; start[buckets] = n
-__global__ void k_starts(ClusterArgs a, const int* excl, const int* block_sum, int64_t buckets) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < buckets) a.start[b] = excl[b] + block_sum[b / kCT];
-  if (b == buckets) a.start[b] = (int)a.n;
+// start[b] = exclusive scan of the counts; start[buckets] = n.  One block per
+// scan tile, which sums the tiles before its own itself.
+__global__ void __launch_bounds__(kCT) k_starts(ClusterArgs a, const int* excl, const int* tile_sum, int64_t buckets) {
+  __shared__ int red[kCT / 32];
+  int sum = 0;
+  for (int t = threadIdx.x; t < (int)blockIdx.x; t += kCT) sum += tile_sum[t];
+  sum = __reduce_add_sync(kFull, sum);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  int base = 0;
+#pragma unroll
+  for (int w = 0; w < kCT / 32; ++w) base += red[w];
+  for (int k = 0; k < kScanPer; ++k) {
+    const int64_t b = (int64_t)blockIdx.x * kScanTile + k * kCT + threadIdx.x;
+    if (b < buckets) a.start[b] = excl[b] + base;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.start[buckets] = (int)a.n;
 }
 
+// Also sets the bucket roots to kNoCore, in the memory of the bucket counts,
+// which the starts have replaced by now.
 template <int DIM>
-__global__ void k_scatter(ClusterArgs a) {
+__global__ void k_scatter(ClusterArgs a, int64_t buckets) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int64_t b = i; b < buckets; b += (int64_t)gridDim.x * blockDim.x) a.broot[b] = kNoCore;
   if (i >= a.n) return;
   const int2 bs = a.bslot[i];
   const int pos = a.start[bs.x] + bs.y;
@@ -309,6 +333,7 @@ __global__ void k_core(ClusterArgs a) {
   a.core[p] = core;
   a.parent[s] = (int)s;
   a.cmin[s] = 0x7fffffff;
+  a.tally[s] = make_int2(0, 0);
 }
 
 // Root of x: parents always point to smaller positions, so the walk ends.
@@ -614,54 +639,98 @@ struct CountValue {
   const int* count;
   __device__ int operator()(int64_t i) const { return count[i]; }
 };
+struct TallyCount {
+  const int2* tally;
+  __device__ int operator()(int64_t i) const { return tally[i].x; }
+};
 struct RootFlag {  // 1 for the root (smallest core index) of each component
   const uint8_t* core;
   const int* root;
   __device__ int operator()(int64_t i) const { return core[i] && root[i] == (int)i ? 1 : 0; }
 };
 
-template <typename Value>
-__global__ void k_scan_blocks(Value value, int64_t len, int* excl, int* block_sum) {
-  __shared__ int s[kCT];
-  const int64_t i = (int64_t)blockIdx.x * kCT + threadIdx.x;
-  const int v = i < len ? value(i) : 0;
-  s[threadIdx.x] = v;
-  __syncthreads();
-  for (int d = 1; d < kCT; d <<= 1) {
-    const int t = threadIdx.x >= d ? s[threadIdx.x - d] : 0;
-    __syncthreads();
-    s[threadIdx.x] += t;
-    __syncthreads();
+// exclusive scan of v over the block, whose total is left in *total
+template <int T>
+__device__ __forceinline__ int block_scan(int v, int* red, int* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int incl = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int t = __shfl_up_sync(kFull, incl, d);
+    if (lane >= d) incl += t;
   }
-  if (i < len) excl[i] = s[threadIdx.x] - v;  // exclusive within the block
-  if (threadIdx.x == kCT - 1) block_sum[blockIdx.x] = s[kCT - 1];
+  if (lane == 31) red[warp] = incl;
+  __syncthreads();
+  int base = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < T / 32; ++w) {
+    base += w < warp ? red[w] : 0;
+    all += red[w];
+  }
+  *total = all;
+  return base + incl - v;
 }
 
-// One block: exclusive scan of the block sums (nb <= kCT * kSumsPerThread).
-__global__ void k_scan_sums(int* block_sum, int nb, int* total) {
-  __shared__ int s[kCT];
-  int loc[kSumsPerThread];
-  int run = 0;
+// One tile of kScanTile values per block: exclusive sums within the tile, and
+// the tile's total.
+template <typename Value>
+__global__ void __launch_bounds__(kCT) k_scan_tiles(Value value, int64_t len, int* excl, int* tile_sum) {
+  __shared__ int red[kCT / 32];
+  const int64_t i0 = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
+  int v[kScanPer], sum = 0, total;
+#pragma unroll
+  for (int k = 0; k < kScanPer; ++k) {
+    v[k] = i0 + k < len ? value(i0 + k) : 0;
+    sum += v[k];
+  }
+  int run = block_scan<kCT>(sum, red, &total);
+#pragma unroll
+  for (int k = 0; k < kScanPer; ++k) {
+    if (i0 + k < len) excl[i0 + k] = run;
+    run += v[k];
+  }
+  if (threadIdx.x == 0) tile_sum[blockIdx.x] = total;
+}
+
+// One block: exclusive scan of the tile sums (nb <= kCT * kSumsPerThread).
+__global__ void __launch_bounds__(kCT) k_scan_sums(int* tile_sum, int nb, int* total) {
+  __shared__ int red[kCT / 32];
+  int v[kSumsPerThread], sum = 0, all;
+#pragma unroll
   for (int k = 0; k < kSumsPerThread; ++k) {
     const int idx = threadIdx.x * kSumsPerThread + k;
-    loc[k] = idx < nb ? block_sum[idx] : 0;
-    run += loc[k];
+    v[k] = idx < nb ? tile_sum[idx] : 0;
+    sum += v[k];
   }
-  s[threadIdx.x] = run;
-  __syncthreads();
-  for (int d = 1; d < kCT; d <<= 1) {
-    const int t = threadIdx.x >= d ? s[threadIdx.x - d] : 0;
-    __syncthreads();
-    s[threadIdx.x] += t;
-    __syncthreads();
-  }
-  int base = s[threadIdx.x] - run;
+  int run = block_scan<kCT>(sum, red, &all);
+#pragma unroll
   for (int k = 0; k < kSumsPerThread; ++k) {
     const int idx = threadIdx.x * kSumsPerThread + k;
-    if (idx < nb) block_sum[idx] = base;
-    base += loc[k];
+    if (idx < nb) tile_sum[idx] = run;
+    run += v[k];
   }
-  if (threadIdx.x == kCT - 1 && total) *total = s[kCT - 1];
+  if (threadIdx.x == 0 && total) *total = all;
+}
+
+// One block: the CSR offsets of up to kOffsetsMax clusters.
+constexpr int kOT = 1024, kOPer = 4, kOffsetsMax = kOT * kOPer;
+__global__ void __launch_bounds__(kOT) k_scan_offsets(const int2* tally, int nc, int* offsets) {
+  __shared__ int red[kOT / 32];
+  int v[kOPer], sum = 0, all;
+#pragma unroll
+  for (int k = 0; k < kOPer; ++k) {
+    const int c = threadIdx.x * kOPer + k;
+    v[k] = c < nc ? tally[c].x : 0;
+    sum += v[k];
+  }
+  int run = block_scan<kOT>(sum, red, &all);
+#pragma unroll
+  for (int k = 0; k < kOPer; ++k) {
+    const int c = threadIdx.x * kOPer + k;
+    if (c < nc) offsets[c] = run;
+    run += v[k];
+  }
+  if (threadIdx.x == 0) offsets[nc] = all;
 }
 
 // Labels, the points per cluster, the noise count and the sort keys of the
@@ -669,7 +738,7 @@ __global__ void k_scan_sums(int* block_sum, int nb, int* total) {
 // per sorted position, so the lanes of a warp mostly share a cluster and
 // add to its count once.
 __global__ void k_label(ClusterArgs a, const int* root, const int* flag_scan, const int* block_sum, int* labels,
-                        int* counts, int* noise, unsigned long long* keys, int64_t n_pad) {
+                        int2* tally, int* noise, unsigned long long* keys, int64_t n_pad) {
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int lab = -2;  // past the end
   if (s < a.n) {
@@ -678,7 +747,7 @@ __global__ void k_label(ClusterArgs a, const int* root, const int* flag_scan, co
     int r = root[i];
     if (r >= 0) {
       if (!a.core[i]) r = root[r];  // a border point's core neighbour -> its root
-      lab = flag_scan[r] + block_sum[r / kCT];
+      lab = flag_scan[r] + block_sum[r / kScanTile];
     }
     labels[i] = lab;
     keys[i] = ((unsigned long long)(uint32_t)(lab >= 0 ? lab : 0x7fffffff) << 32) | (unsigned long long)i;
@@ -687,15 +756,15 @@ __global__ void k_label(ClusterArgs a, const int* root, const int* flag_scan, co
   }
   const unsigned peers = __match_any_sync(kFull, lab);
   const int lane = threadIdx.x & 31;
-  if (lab >= 0 && (peers & ((1u << lane) - 1u)) == 0u) atomicAdd(&counts[lab], __popc(peers));
+  if (lab >= 0 && (peers & ((1u << lane) - 1u)) == 0u) atomicAdd(&tally[lab].x, __popc(peers));
   const unsigned nz = __ballot_sync(kFull, lab == -1);
   if (lane == 0 && nz) atomicAdd(noise, __popc(nz));
 }
 
 // the largest cluster (clusters 0 .. *total - 1)
-__global__ void k_maxcount(const int* counts, int64_t n, const int* total, int* maxc) {
+__global__ void k_maxcount(const int2* tally, int64_t n, const int* total, int* maxc) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int v = c < n && c < *total ? counts[c] : 0;
+  const int v = c < n && c < *total ? tally[c].x : 0;
   const int m = __reduce_max_sync(kFull, v);
   if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(maxc, m);
 }
@@ -703,21 +772,21 @@ __global__ void k_maxcount(const int* counts, int64_t n, const int* total, int* 
 // ---- the CSR: clusters placed by offsets, each cluster's indices sorted -----------
 __global__ void k_offsets(const int* excl, const int* block_sum, int n_clusters, int n_clustered, int* offsets) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < n_clusters) offsets[c] = excl[c] + block_sum[c / kCT];
+  if (c < n_clusters) offsets[c] = excl[c] + block_sum[c / kScanTile];
   if (c == n_clusters) offsets[c] = n_clustered;
 }
 
 // places each clustered point in its cluster's range (in no particular
 // order: k_segsort orders it); by sorted position, one atomic per cluster
 // and warp
-__global__ void k_place(const int* sidx, const int* labels, int64_t n, const int* offsets, int* cursor, int* perm) {
+__global__ void k_place(const int* sidx, const int* labels, int64_t n, const int* offsets, int2* tally, int* perm) {
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int i = s < n ? sidx[s] : -1;
   const int lab = i >= 0 ? labels[i] : -1;
   const unsigned peers = __match_any_sync(kFull, lab);
   const int lane = threadIdx.x & 31, lead = __ffs(peers) - 1;
   int base = 0;
-  if (lab >= 0 && lane == lead) base = atomicAdd(&cursor[lab], __popc(peers));
+  if (lab >= 0 && lane == lead) base = atomicAdd(&tally[lab].y, __popc(peers));
   base = __shfl_sync(kFull, base, lead);
   if (lab >= 0) perm[offsets[lab] + base + __popc(peers & ((1u << lane) - 1u))] = i;
 }
@@ -828,12 +897,13 @@ __global__ void k_gather(const int* perm, int64_t m, const float* s0, float* d0,
 }
 
 inline unsigned grid_for(int64_t n) { return (unsigned)((n + kCT - 1) / kCT); }
+inline unsigned tiles_for(int64_t n) { return (unsigned)((n + kScanTile - 1) / kScanTile); }
 
 // buckets: a power of two >= 4 n (fewer far cells sharing a bucket), at
 // least 64 (two bits or more per gridded component) and at most what the
 // one-block scan takes, which is >= n; n_pad: the bitonic length, a power of
 // two >= n
-constexpr int64_t kMaxBuckets = (int64_t)kCT * kSumsPerThread * kCT;
+constexpr int64_t kMaxBuckets = (int64_t)kScanTile * kCT * kSumsPerThread;
 void table_sizes(int64_t n, int64_t* buckets, int64_t* n_pad) {
   int64_t b = 64, p = 1;
   while (b < 4 * n && b < kMaxBuckets) b <<= 1;
@@ -845,20 +915,16 @@ void table_sizes(int64_t n, int64_t* buckets, int64_t* n_pad) {
 template <int DIM>
 cudaError_t launch_grid_phase(ClusterArgs& a, int64_t buckets, int* excl, int* block_sum, int* root,
                               cudaStream_t s) {
-  const unsigned nbb = grid_for(buckets);
+  const unsigned tiles = tiles_for(buckets);
   k_grid<DIM><<<grid_for(a.n), kCT, 0, s>>>(a);
-  k_scan_blocks<<<nbb, kCT, 0, s>>>(CountValue{a.count}, buckets, excl, block_sum);
-  k_scan_sums<<<1, kCT, 0, s>>>(block_sum, (int)nbb, nullptr);
-  k_starts<<<grid_for(buckets + 1), kCT, 0, s>>>(a, excl, block_sum, buckets);
-  k_scatter<DIM><<<grid_for(a.n), kCT, 0, s>>>(a);
+  k_scan_tiles<<<tiles, kCT, 0, s>>>(CountValue{a.count}, buckets, excl, block_sum);
+  k_starts<<<tiles, kCT, 0, s>>>(a, excl, block_sum, buckets);
+  k_scatter<DIM><<<grid_for(a.n), kCT, 0, s>>>(a, buckets);
   k_core<DIM><<<grid_for(a.n), kCT, 0, s>>>(a);
   k_link_blocks<DIM><<<(unsigned)((a.n + kLT - 1) / kLT), kLT, 0, s>>>(a);
-  // the bucket counts are consumed by now: their memory holds the bucket roots
-  cudaError_t e = cudaMemsetAsync(a.broot, 0xfe, (size_t)buckets * 4, s);
-  if (e != cudaSuccess) return e;
   k_bucket_roots<<<grid_for(a.n), kCT, 0, s>>>(a);
   k_union<DIM, true><<<grid_for((a.n + kSample - 1) / kSample * kUGSampled), kCT, 0, s>>>(a);
-  e = cudaMemsetAsync(a.broot, 0xfe, (size_t)buckets * 4, s);
+  const cudaError_t e = cudaMemsetAsync(a.broot, 0xfe, (size_t)buckets * 4, s);
   if (e != cudaSuccess) return e;
   k_bucket_roots<<<grid_for(a.n), kCT, 0, s>>>(a);
   k_union<DIM, false><<<grid_for(a.n * kUGRest), kCT, 0, s>>>(a);
@@ -872,20 +938,20 @@ cudaError_t launch_grid_phase(ClusterArgs& a, int64_t buckets, int* excl, int* b
 size_t cluster_scratch_bytes(int64_t n) {
   int64_t buckets, pad;
   table_sizes(n, &buckets, &pad);
-  const int64_t nbb = (buckets + kCT - 1) / kCT;
+  const int64_t nbb = (buckets + kScanTile - 1) / kScanTile;
   // thirteen sub-buffers, each start rounded up to 256 bytes
   return (size_t)pad * 8 + (size_t)buckets * 12 + 4 + (size_t)nbb * 4 + (size_t)n * (8 + 16 + 4 + 1 + 1 + 4 + 4) +
          64 + 13 * 256;
 }
 
-int64_t cluster_max_points() { return (int64_t)kCT * kSumsPerThread * kCT; }
+int64_t cluster_max_points() { return kMaxBuckets; }
 
 cudaError_t launch_cluster(const float* feat, int64_t n, int dim, double eps, int min_pts, void* scratch,
                            int* labels, int* perm, int* offsets, int max_clusters, int* n_clusters_host,
-                           int* err_host, cudaStream_t s) {
+                           int* err_host, int* h, cudaStream_t s) {
   int64_t buckets, pad;
   table_sizes(n, &buckets, &pad);
-  const int64_t nbb = (buckets + kCT - 1) / kCT;
+  const int64_t nbb = (buckets + kScanTile - 1) / kScanTile;
   char* b = (char*)scratch;
   auto take = [&](size_t bytes) {
     char* p = b;
@@ -896,6 +962,7 @@ cudaError_t launch_cluster(const float* feat, int64_t n, int dim, double eps, in
   float4* sfeat = (float4*)take((size_t)n * 16);
   int2* bslot = (int2*)take((size_t)n * 8);
   int* count = (int*)take((size_t)buckets * 4);
+  int* small = (int*)take(64);  // err, clusters, noise, largest cluster; right after the counts, zeroed with them
   int* start = (int*)take((size_t)buckets * 4 + 4);
   // the bucket scan, then the component minima, then the root-flag scan (n <= buckets)
   int* excl = (int*)take((size_t)buckets * 4);
@@ -905,7 +972,6 @@ cudaError_t launch_cluster(const float* feat, int64_t n, int dim, double eps, in
   int* root = (int*)take((size_t)n * 4);
   uint8_t* score = (uint8_t*)take((size_t)n);
   uint8_t* core = (uint8_t*)take((size_t)n);
-  int* small = (int*)take(64);  // err, total, noise
 
   ClusterArgs a;
   a.feat = feat;
@@ -944,6 +1010,7 @@ cudaError_t launch_cluster(const float* feat, int64_t n, int dim, double eps, in
   a.count = count;
   a.start = start;
   a.bslot = bslot;
+  a.tally = bslot;
   a.sfeat = sfeat;
   a.sidx = sidx;
   a.sbkt = (uint32_t*)keys;  // the keys are written once no kernel needs the buckets any more
@@ -955,8 +1022,7 @@ cudaError_t launch_cluster(const float* feat, int64_t n, int dim, double eps, in
   a.err = small;
 
   cudaError_t e;
-  if ((e = cudaMemsetAsync(count, 0, (size_t)buckets * 4, s)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(small, 0, 64, s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(count, 0, (size_t)buckets * 4 + 64, s)) != cudaSuccess) return e;
   switch (dim) {
     case 1: e = launch_grid_phase<1>(a, buckets, excl, block_sum, root, s); break;
     case 2: e = launch_grid_phase<2>(a, buckets, excl, block_sum, root, s); break;
@@ -965,32 +1031,28 @@ cudaError_t launch_cluster(const float* feat, int64_t n, int dim, double eps, in
     default: return cudaErrorInvalidValue;
   }
   if (e != cudaSuccess) return e;
-  // per-cluster counts and placement cursors in the bucket slots (dead after k_scatter)
-  int* counts = (int*)bslot;
-  int* cursor = counts + n;
-  if ((e = cudaMemsetAsync(counts, 0, (size_t)n * 8, s)) != cudaSuccess) return e;
-  const int64_t nb = (n + kCT - 1) / kCT;
-  k_scan_blocks<<<(unsigned)nb, kCT, 0, s>>>(RootFlag{core, root}, n, excl, block_sum);
-  k_scan_sums<<<1, kCT, 0, s>>>(block_sum, (int)nb, small + 1);
-  k_label<<<grid_for(pad), kCT, 0, s>>>(a, root, excl, block_sum, labels, counts, small + 2, keys, pad);
-  k_maxcount<<<grid_for(n), kCT, 0, s>>>(counts, n, small + 1, small + 3);
+  k_scan_tiles<<<tiles_for(n), kCT, 0, s>>>(RootFlag{core, root}, n, excl, block_sum);
+  k_scan_sums<<<1, kCT, 0, s>>>(block_sum, (int)tiles_for(n), small + 1);
+  k_label<<<grid_for(pad), kCT, 0, s>>>(a, root, excl, block_sum, labels, a.tally, small + 2, keys, pad);
+  k_maxcount<<<grid_for(n), kCT, 0, s>>>(a.tally, n, small + 1, small + 3);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  int h[4] = {0, 0, 0, 0};  // err, clusters, noise, largest cluster
-  if ((e = cudaMemcpyAsync(h, small, sizeof(h), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+  // err, clusters, noise, largest cluster, into page-locked memory
+  if ((e = cudaMemcpyAsync(h, small, 4 * sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
   *err_host = h[0];
   *n_clusters_host = h[1];
   if (h[0] || h[1] > max_clusters) return cudaSuccess;  // the caller reports it; no CSR written
   const int nc = h[1], n_clustered = (int)(n - h[2]);
   if (h[3] <= kSegMax) {
-    if (nc > 0) {
-      const int64_t nbc = (nc + kCT - 1) / kCT;
-      k_scan_blocks<<<(unsigned)nbc, kCT, 0, s>>>(CountValue{counts}, nc, excl, block_sum);
-      k_scan_sums<<<1, kCT, 0, s>>>(block_sum, (int)nbc, nullptr);
+    if (nc <= kOffsetsMax) {
+      k_scan_offsets<<<1, kOT, 0, s>>>(a.tally, nc, offsets);
+    } else {
+      k_scan_tiles<<<tiles_for(nc), kCT, 0, s>>>(TallyCount{a.tally}, nc, excl, block_sum);
+      k_scan_sums<<<1, kCT, 0, s>>>(block_sum, (int)tiles_for(nc), nullptr);
+      k_offsets<<<grid_for((int64_t)nc + 1), kCT, 0, s>>>(excl, block_sum, nc, n_clustered, offsets);
     }
-    k_offsets<<<grid_for((int64_t)nc + 1), kCT, 0, s>>>(excl, block_sum, nc, n_clustered, offsets);
     if (nc > 0) {
-      k_place<<<grid_for(n), kCT, 0, s>>>(sidx, labels, n, offsets, cursor, perm);
+      k_place<<<grid_for(n), kCT, 0, s>>>(sidx, labels, n, offsets, a.tally, perm);
       k_segsort<<<(unsigned)nc, kSegT, 0, s>>>(perm, offsets);
     }
   } else {  // a cluster too large for one block: sort all (cluster, index) keys
