@@ -25,14 +25,15 @@
 // neighbour, walk alone (batched loads) when their neighbourhood is small
 // and with the whole warp (coalesced tiles, ballots) when it is large.  Then
 // a lock-free union-find over core-core neighbour pairs on sorted positions:
-// a near-neighbour linking pass within blocks first, a root recorded
-// per bucket, and a full pass, eight lanes per point, that skips buckets
-// already in the point's set; it links the larger root under the smaller.  An atomic
-// minimum per component gives its smallest core index; a device-wide scan
-// numbers the clusters.  The CSR:
-// per-cluster counts, offsets by a scan, placement, and a shared-memory sort
-// of each cluster's indices (a global bitonic sort of (cluster, index) keys
-// when a cluster exceeds one block's capacity).
+// near neighbours are linked within blocks in shared memory first; then a root
+// is recorded per bucket and a full pass, which skips buckets already in the
+// point's set, runs for every kSample-th point (a warp each) and, with the
+// bucket roots taken anew, for the rest; it links the larger root under the
+// smaller.  An atomic minimum per component gives its smallest core index; a
+// device-wide scan numbers the clusters.  The CSR: per-cluster counts, offsets
+// by a scan (one block for up to kOffsetsMax clusters), placement, and a
+// shared-memory sort of each cluster's indices (a global bitonic sort of
+// (cluster, index) keys when a cluster exceeds one block's capacity).
 // Every loop is bounded by the input size; the union retry loop has an
 // explicit cap that raises an error flag instead of spinning.
 #include <cstdint>

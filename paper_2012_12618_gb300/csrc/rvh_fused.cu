@@ -1,16 +1,17 @@
 // Fused persistent kernel: per cluster, FP32 and FP64 rows -> counter-RNG
-// minimal sets -> FP32 solve with error bound (refined in FP64 residuals when
-// ill-conditioned) -> FP32 scoring pass (upper-bound counts) -> exact counts,
-// in index order, of the trials that can still win (FP64 only inside the
-// error band) -> lowest-index argmax -> FP64 inlier mask and normal-equation
-// refine -> heading.  Sec. III-A (Alg. 1, Eq. 4) and Sec. III-B (Eq. LSQ_eq,
+// minimal sets -> FP32 solve with error bound (refined when ill-conditioned:
+// 3D with residuals in pairs of FP32, 2D in FP64) -> FP32 scoring pass
+// (upper-bound counts; in stages that drop trials the lead's residuals rule
+// out) -> exact counts, best bound first, of the trials that can still win
+// (FP64 only inside the error band) -> lowest-index argmax -> FP64 inlier mask
+// and normal-equation refine -> heading.  Sec. III-A (Alg. 1, Eq. 4) and Sec. III-B (Eq. LSQ_eq,
 // Eq. eq:LSQPerCluster, Alg. 2) of arXiv 2012.12618.
 //
 // Parallel mapping (GB300-first, not the paper's thread-per-trial): clusters
 // are work items taken by persistent CTAs from an LPT-ordered list; inside a
 // cluster, trials map to warps/lanes and points to lanes, with the cluster's
-// FP32 rows staged in shared memory and its FP64 rows in L1/L2-resident
-// global scratch.
+// FP32 rows staged in shared memory (what exceeds it in global scratch) and its
+// FP64 rows in L1/L2-resident global scratch.
 #include <cstdint>
 #include <type_traits>
 #include <cuda_runtime.h>
