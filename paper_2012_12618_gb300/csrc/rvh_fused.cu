@@ -266,6 +266,21 @@ __device__ __forceinline__ HoldRange hold_range(const DirRange& g, float4 lead, 
   return h;
 }
 
+// The red_ arrays carry values between warps.  Between the reads of one use
+// and the writes of the next lies a barrier, each time:
+//   red_i  medians (write, barrier, read, barrier); the staged pass's tops
+//          (then the lead pass's barriers); prune_list (a barrier at its end);
+//          the mask pass's inlier counts (a barrier at its end)
+//   red_c  the staged pass's counts of the lead, while warps may still read the
+//          tops in red_i (a barrier after them); the mask pass's changed
+//          entries (a barrier at its end)
+//   red_u  block_best: count_trial's barriers before the next, or the one after the loop
+//   red_v  block_sum2: a barrier between its two uses in a count, and at count_trial's end
+//   red_f  block_max_float, once per cluster
+//   red_d  the line model's ranges (write, barrier, read, barrier), then the direction
+//          range, read by thread 0 before the trials' barrier
+//   red_t  the mask pass's sums, read after its last barrier and written after
+//          the first one of the next pass
 struct ClusterShared {
   unsigned long long best;
   float4 win;      // winner's FP32 record
@@ -280,7 +295,7 @@ struct ClusterShared {
   double cv64[3];             // FP64 velocity of the trial being counted (when it has band points)
   double win_v64[3];          // FP64 velocity of the current winner (valid if win_has_v64)
   int win_has_v64;
-  int red_c[kWarps];          // changed mask entries (local-optimisation rounds)
+  int red_c[kWarps];
   double lo_v[3];             // least-squares velocity of the current inlier set
   float4 lo_hy;               // its FP32 record (-X, -Y, -Z, thi) and lower threshold
   float lo_tlo;
@@ -1214,7 +1229,7 @@ __device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, co
       }
     }
     cnt = __reduce_add_sync(0xffffffffu, cnt);
-    if (lane == 0) cs.red_i[warp] = (int)cnt;
+    if (lane == 0) cs.red_c[warp] = (int)cnt;  // not red_i: a warp may still be reading the tops there
     __syncthreads();
     if (warp < 1 + NH) {  // warp 1: outside, the others: inside, a half of a2 each
       unsigned* h = warp == 1 ? cs.lead_out : cs.lead_in + (warp >> 1) * (kTanBins + 1);
@@ -1246,7 +1261,7 @@ __device__ __forceinline__ unsigned long long staged_pass(const FrameDesc& a, co
         if (lane == 31) put(kTanBins, incl.x, incl.y);
       }
     } else if (warp == 3) {
-      const unsigned v = __reduce_add_sync(0xffffffffu, lane < kWarps ? (unsigned)cs.red_i[lane] : 0u);
+      const unsigned v = __reduce_add_sync(0xffffffffu, lane < kWarps ? (unsigned)cs.red_c[lane] : 0u);
       if (lane == 0) cs.lead_cnt = v;
     }
     __syncthreads();
