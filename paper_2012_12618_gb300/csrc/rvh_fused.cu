@@ -1675,6 +1675,16 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
   stage_done(4);
 }
 
+// Clusters beyond the shared-memory rows under an extension.  Out of line:
+// beside the inlined copy for the others, the 2D kernel's path for those
+// spilled 416 bytes (96 so).  Dense 2D frame, us per pass: adaptive count 157
+// -> 152, local optimisation 358 -> 350, line model 352 -> 334.
+template <int DIM, bool EXT>
+__device__ __noinline__ void process_large(const FrameDesc& a, const Smem& S, ClusterShared& cs, int ci, int hchunk,
+                                           int pw, int prune, int frame, FinishRec* fq, int* fq_n, int row_cap) {
+  process_cluster<DIM, false, EXT>(a, S, cs, ci, hchunk, pw, prune, frame, fq, fq_n, nullptr, row_cap);
+}
+
 // EXT = true: the instantiation with the extensions of the method (the
 // local-optimisation rounds and the adaptive trial count), launched only for
 // batches that ask for one of them; the default instantiation carries no
@@ -1764,6 +1774,8 @@ __global__ void __launch_bounds__(kThreads, RVH_MIN_BLOCKS) fused_kernel(const _
     const int cap = smem_row_capacity(DIM, a.nmax_smem);
     if (e - o <= (int64_t)cap || e < o) {
       process_cluster<DIM, true, EXT>(F, S, cs, ci, a.hchunk, a.pw, a.prune, fc.x, fq, &fq_n, cta_pre, cap);
+    } else if constexpr (EXT) {
+      process_large<DIM, EXT>(F, S, cs, ci, a.hchunk, a.pw, a.prune, fc.x, fq, &fq_n, cap & ~31);
     } else {
       process_cluster<DIM, false, EXT>(F, S, cs, ci, a.hchunk, a.pw, a.prune, fc.x, fq, &fq_n, cta_pre, cap & ~31);
     }
