@@ -178,6 +178,9 @@ constexpr float kRowRel3 = 2.0f * 0x1p-22f + 2.0f * 0x1p-24f;  // products cos t
 constexpr float kSafety = 1.0f + 0x1p-14f;   // covers second-order terms and bound roundings
 constexpr float kTiny = 0x1p-120f;           // absolute slack for underflow
 constexpr float kBandFloor = 1e-5f;          // minimum half-width of the FP64 band (m/s)
+// Largest half-width of a normal record: the band is at least 2u (wmax + |X|),
+// so |w| and |X| stay below 2^59, residuals below 2^62 and their squares finite.
+constexpr float kBandMax = 0x1p36f;
 // |det32 - det64| over unit rows: (2 rho + 2u)(1 + 1e-4) for 2D,
 // sqrt(3)(3 rho3 + 5u) for 3D, rounded up, plus the FP64 rounding of det64.
 constexpr float kDetErr2 = 5.98e-7f;
@@ -404,7 +407,7 @@ __device__ __forceinline__ Hyp32 hyp_f32(float4 p, float4 q, float4 r, const See
                                          float wmax, float acc, float rej, TauPair tau) {
   Hyp32 h;
   h.nx = h.ny = h.nz = 0.0f;
-  h.thi = __int_as_float(0x7fc00000);  // NaN: never counted
+  h.thi = __int_as_float(0x7fc00000);  // NaN: no threshold (rejected)
   h.tlo = -1.0f;
   h.refined = 0;
   float d;
@@ -456,7 +459,7 @@ __device__ __forceinline__ Hyp32 hyp_f32(float4 p, float4 q, float4 r, const See
   h.nx = -X[0];
   h.ny = -X[1];
   h.nz = -X[2];
-  if (!(b < 1e30f) || !(fabsf(X[0]) < 1e30f) || !(fabsf(X[1]) < 1e30f) || !(fabsf(X[2]) < 1e30f) ||
+  if (!(b < kBandMax) || !(fabsf(X[0]) < 1e30f) || !(fabsf(X[1]) < 1e30f) || !(fabsf(X[2]) < 1e30f) ||
       !(ad > 2.0f * eD)) {
     h.kind = kHypExactOnly;
     h.thi = __int_as_float(0x7f800000);  // +inf: nothing certainly out

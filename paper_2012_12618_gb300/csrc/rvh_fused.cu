@@ -413,7 +413,7 @@ __device__ __forceinline__ Hyp32 line_record(const double v[3], double T) {
   h.kind = kHypNormal;
   h.thi = __double2float_ru(hi);
   h.nz = h.tlo = lo >= 0.0 ? __double2float_rd(lo) : -1.0f;
-  if (!(hi < 1e30) || !(am < 1e30) || !(ac < 1e30)) {
+  if (!(hi < 1e30) || !(am < 0x1p60) || !(ac < 0x1p60)) {  // residuals below 2^62: finite squares
     h.kind = kHypExactOnly;
     h.thi = __int_as_float(0x7f800000);
     h.nz = h.tlo = -1.0f;

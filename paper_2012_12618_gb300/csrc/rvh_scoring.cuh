@@ -124,9 +124,10 @@ __device__ __forceinline__ int sign_count(uint32_t acc) {
 
 // -C with C the smallest float above thi^2 rounded up: C > thi^2, so
 // r^2 < C for every |r| <= thi, and r^2 < C holds beyond thi only for r^2
-// within two ulps of thi^2.
+// within two ulps of thi^2.  A square beyond FP32 (thi up to infinity) gives
+// C = inf, which holds every r^2: normal records have finite ones (kBandMax).
 __device__ __forceinline__ float neg_count_bound(float thi) {
-  return -__uint_as_float(__float_as_uint(__fmul_ru(thi, thi)) + 1u);
+  return -__uint_as_float(min(__float_as_uint(__fmul_ru(thi, thi)) + 1u, 0x7f800000u));
 }
 
 // HPL trial records of one lane in packed registers: (-X, -X), (-Y, -Y),
@@ -135,7 +136,7 @@ template <int HPL>
 struct LaneTrials {
   unsigned long long nx[HPL], ny[HPL], nz[HPL], nc[HPL];
   uint32_t acc[HPL];
-  // record (-X, -Y, -Z, thi) into slot m; a NaN thi never counts
+  // record (-X, -Y, -Z, thi) into slot m; the counts of a NaN thi mean nothing
   __device__ __forceinline__ void load(int m, float4 v) {
     nx[m] = pack2(v.x, v.x);
     ny[m] = pack2(v.y, v.y);
