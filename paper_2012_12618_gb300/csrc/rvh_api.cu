@@ -182,7 +182,10 @@ struct rvh_ctx {
   int* cl_readback = nullptr;  // page-locked, 4 ints
   cudaEvent_t last_done = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-  unsigned long long* stats_d = nullptr;
+  // The launch counters' three copies, zeroed when the context is made, so that
+  // no call, whatever becomes of it or of the scratch, leaves them unset.
+  void* counters = nullptr;
+  unsigned long long* stats_d = nullptr;  // the copy the last launch counted in
   int stats_slot = 0;  // the counters' clean copy (launch_graph): used by the next call, which cleans the other
   bool have_launch = false;
   rvh_stats last{};
@@ -455,6 +458,17 @@ int rvh_create(rvh_ctx** out, int device, size_t mem_budget_bytes) {
     c->trig = (double2*)p;
   }
   {
+    int rc = ctx_alloc(c, &c->counters, 3 * kStatsBytes);
+    if (rc == RVH_OK && (cudaMemsetAsync(c->counters, 0, 3 * kStatsBytes, c->stream) != cudaSuccess ||
+                         cudaStreamSynchronize(c->stream) != cudaSuccess))
+      rc = fail(RVH_ECUDA, "counters not set");
+    if (rc != RVH_OK) {
+      cudaGetLastError();
+      rvh_destroy(c);
+      return rc;
+    }
+  }
+  {
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) == cudaSuccess)
       c->tune_prefix = std::string(prop.name) + "|" + std::to_string(c->sms) + "|";
@@ -476,6 +490,7 @@ void rvh_destroy(rvh_ctx* ctx) {
   if (ctx->scratch) ctx_free(ctx, ctx->scratch, ctx->scratch_bytes);
   if (ctx->cl_scratch) ctx_free(ctx, ctx->cl_scratch, ctx->cl_scratch_bytes);
   if (ctx->cl_readback) cudaFreeHost(ctx->cl_readback);
+  if (ctx->counters) ctx_free(ctx, ctx->counters, 3 * kStatsBytes);
   if (ctx->trig) ctx_free(ctx, ctx->trig, sizeof(double2) * kTrigSize);
   cudaEventDestroy(ctx->last_done);
   cudaEventDestroy(ctx->ev0);
@@ -607,7 +622,6 @@ struct Staged {
   char* base;
   int2* worklist;
   int* counter;
-  unsigned long long* stats;
   void* rows;               // float4[n_points] (fused) or double[4 n_points] (baseline)
   double4_32a* rows64;      // double4_32a[n_points] (fused)
   double4_32a* cta_rows64;  // double4_32a[resident CTAs * max over dims of cta_slot_stride] (fused)
@@ -653,7 +667,6 @@ static int stage(rvh_ctx* ctx, const rvh_frame* f, const rvh_params* p, rvh_resu
     off += align_up(bytes);
     return o;
   };
-  const size_t o_stats = take(3 * kStatsBytes);  // first: its place does not depend on the frame
   const size_t o_work = take(sizeof(int2) * (size_t)std::max(nc, 1));
   const size_t o_ctr = take(64);
   const size_t o_rows = take((fused ? sizeof(float4) : 4 * sizeof(double)) * (size_t)std::max<int64_t>(np, 1));
@@ -685,13 +698,11 @@ static int stage(rvh_ctx* ctx, const rvh_frame* f, const rvh_params* p, rvh_resu
     int rc = ctx_alloc(ctx, &ctx->scratch, want);
     if (rc) return rc;
     ctx->scratch_bytes = want;
-    RVH_CUDA(cudaMemsetAsync(ctx->scratch, 0, 3 * kStatsBytes, s));
   }
   char* b = (char*)ctx->scratch;
   st.base = b;
   st.worklist = (int2*)(b + o_work);
   st.counter = (int*)(b + o_ctr);
-  st.stats = (unsigned long long*)(b + o_stats);
   st.rows = b + o_rows;
   st.rows64 = fused ? (double4_32a*)(b + o_rows64) : nullptr;
   st.cta_rows64 = fused ? (double4_32a*)(b + o_cta64) : nullptr;
@@ -753,13 +764,14 @@ int rvh_estimate(rvh_ctx* ctx, const rvh_frame* frame, const rvh_params* params,
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   RVH_CUDA(cudaStreamIsCapturing(s, &cap));
   constexpr size_t kStride = kStatsBytes / sizeof(unsigned long long);
+  unsigned long long* counters = (unsigned long long*)ctx->counters;
   if (ctx->graphs && s != nullptr && cap == cudaStreamCaptureStatusNone) {
-    a.stats = st.stats + (size_t)ctx->stats_slot * kStride;
-    a.stats_next = st.stats + (size_t)(ctx->stats_slot ^ 1) * kStride;
+    a.stats = counters + (size_t)ctx->stats_slot * kStride;
+    a.stats_next = counters + (size_t)(ctx->stats_slot ^ 1) * kStride;
     ctx->stats_d = a.stats;
     rc = launch_graph(ctx, a, params->model_dim, s);
   } else {
-    a.stats = ctx->stats_d = st.stats + 2 * kStride;
+    a.stats = ctx->stats_d = counters + 2 * kStride;
     RVH_CUDA(cudaMemsetAsync(a.stats, 0, sizeof(unsigned long long) * kStatsWords, s));
     rc = launch_batch(ctx, a, params->model_dim, s, ctx->ev0, ctx->ev1);
   }
