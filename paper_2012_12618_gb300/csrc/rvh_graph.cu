@@ -38,8 +38,7 @@ void LaunchGraph::reset() {
 
 cudaError_t LaunchGraph::launch(const FusedArgs& a, int dim, int grid, size_t smem, bool with_work, cudaStream_t s) {
   const bool ext = fused_ext(a);
-  FusedArgs arg = a;  // the node parameters are copied when set
-  void* args[] = {(void*)&arg};
+  void* args[] = {(void*)&a};  // copied when a node's parameters are set
   const cudaKernelNodeParams pf = node_params(fused_kernel_fn(dim, ext), grid, fused_threads(), smem, args);
   const cudaKernelNodeParams pw = node_params(worklist_kernel_fn(), 1, kWorklistThreads, 0, args);
   cudaError_t e = cudaSuccess;
@@ -58,7 +57,13 @@ cudaError_t LaunchGraph::launch(const FusedArgs& a, int dim, int grid, size_t sm
     with_work_ = with_work;
     ++builds;
   } else {
-    const bool same = have_last && last_grid == grid && last_smem == smem && memcmp(&last, &a, sizeof(FusedArgs)) == 0;
+    // A batch with counters (rvh_estimate) never repeats its arguments, as their
+    // two copies take turns: it is neither compared (6.7 KB) nor copied.  Host time
+    // of a call with 64 clusters: a repeated frame 8.65 -> 8.3 us, frames in turn 6.75 -> 6.4.
+    // Two executables, one per copy, need no update for a repeated frame (5.8 us),
+    // but alternating them took 0.5 us more on the device (19.5 -> 20.0 us per pass).
+    const bool same = !a.stats && have_last && last_grid == grid && last_smem == smem &&
+                      memcmp(&last, &a, sizeof(FusedArgs)) == 0;
     if (!same) {
       e = cudaGraphExecKernelNodeSetParams(exec, fused, &pf);
       if (e == cudaSuccess && with_work) e = cudaGraphExecKernelNodeSetParams(exec, work, &pw);
@@ -69,10 +74,10 @@ cudaError_t LaunchGraph::launch(const FusedArgs& a, int dim, int grid, size_t sm
     }
     ++replays;
   }
-  last = a;
+  if (!a.stats) last = a;
+  have_last = !a.stats;
   last_grid = grid;
   last_smem = smem;
-  have_last = true;
   return cudaGraphLaunch(exec, s);
 }
 
