@@ -340,7 +340,9 @@ int rvh_get_stats(rvh_ctx* ctx, rvh_stats* out);
 
 /* Fixes the scoring schedule: points_per_warp in {1, 8, 32} (lanes over points
  * per trial group) and hyps_per_lane in {4, 8}; 0 restores the automatic
- * choice. */
+ * choice.  Every schedule runs four trials per lane (two for the trials that
+ * pruning leaves): hyps_per_lane 8 is accepted, reported in rvh_stats, and
+ * runs as 4. */
 int rvh_set_schedule(rvh_ctx* ctx, int32_t points_per_warp, int32_t hyps_per_lane);
 
 /* Staged scoring with exact pruning (default on): the scoring pass of a
@@ -365,7 +367,7 @@ typedef struct {
 } rvh_schedule;
 
 /* Autotuner: runs the fused kernel on this frame with every scoring schedule
- * (points_per_warp in {1, 8, 32} x hyps_per_lane in {4, 8}), the schedules
+ * (points_per_warp in {1, 8, 32}, hyps_per_lane 4), the schedules
  * taking turns for one untimed and then `reps` timed rounds (CUDA events on
  * the context's stream), and keeps the one with the lowest median time for
  * frames of this model dimension and trial-count bucket (floor(log2) of the

@@ -850,18 +850,19 @@ int rvh_autotune(rvh_ctx* ctx, const rvh_frame* frame, const rvh_params* params,
   int rc = check_args_impl(frame, params, result);
   if (rc) return rc;
   if (frame->n_clusters == 0) return fail(RVH_EINVAL, "empty frame");
-  static const int kCand[6][2] = {{1, 4}, {1, 8}, {8, 4}, {8, 8}, {32, 4}, {32, 8}};
+  static const int kCand[3] = {1, 8, 32};  // points_per_warp; every one runs four trials per lane
   const int save_pw = ctx->pw_fixed, save_hpl = ctx->hpl_fixed;
-  int bpw = 1, bhpl = 4;
+  int bpw = 1;
+  constexpr int bhpl = 4;
   float bms = 1e30f;
   // candidates take turns (round-robin over the repetitions, the first
   // round untimed) so that drifting clocks or caches favour none of them;
   // each is ranked by its median time
-  std::vector<std::vector<float>> times(6);
+  std::vector<std::vector<float>> times(3);
   for (int r = 0; r <= reps && rc == RVH_OK; ++r) {
-    for (int ic = 0; ic < 6 && rc == RVH_OK; ++ic) {
-      ctx->pw_fixed = kCand[ic][0];
-      ctx->hpl_fixed = kCand[ic][1];
+    for (int ic = 0; ic < 3 && rc == RVH_OK; ++ic) {
+      ctx->pw_fixed = kCand[ic];
+      ctx->hpl_fixed = bhpl;
       rc = rvh_estimate(ctx, frame, params, result, nullptr);
       if (rc) break;
       rvh_stats st;
@@ -869,14 +870,13 @@ int rvh_autotune(rvh_ctx* ctx, const rvh_frame* frame, const rvh_params* params,
       if (r > 0) times[ic].push_back(st.kernel_ms);
     }
   }
-  for (int ic = 0; ic < 6 && rc == RVH_OK; ++ic) {
+  for (int ic = 0; ic < 3 && rc == RVH_OK; ++ic) {
     std::vector<float>& t = times[ic];
     std::sort(t.begin(), t.end());
     const float ms = t.size() % 2 ? t[t.size() / 2] : 0.5f * (t[t.size() / 2 - 1] + t[t.size() / 2]);
     if (ms < bms) {
       bms = ms;
-      bpw = kCand[ic][0];
-      bhpl = kCand[ic][1];
+      bpw = kCand[ic];
     }
   }
   ctx->pw_fixed = save_pw;
