@@ -33,7 +33,9 @@
  *   - the pseudo-inverse is taken through the FP64 normal equations of the
  *     inliers; with fewer than k inliers, or |det(A^T A)| <= 1e-12 trace^k,
  *     the winning minimal-set velocity is returned with RVH_STATUS_LSQ_FALLBACK;
- *   - the heading is atan2(vy, vx) in (-pi, pi].
+ *   - the heading is atan2(vy, vx) in (-pi, pi], formed from the normal
+ *     equations beside the velocity: within 3 x 2^-52 rad of the solution's
+ *     angle, so its last bits may differ from atan2 of the returned vy, vx.
  * Every inlier decision, count and winner index equals that of an FP64
  * evaluation of the same formulas: scoring runs in FP32 with a rigorous
  * per-trial error bound, and points whose FP32 residual is within the bound
@@ -160,7 +162,7 @@ typedef struct {
   double* vx;                /* m/s, longitudinal (Sec. III-B) */
   double* vy;                /* m/s, lateral */
   double* vz;                /* m/s, vertical (3D model) */
-  double* heading;           /* rad, atan2(vy, vx) */
+  double* heading;           /* rad, atan2(vy, vx) up to its last bits */
   int32_t* inlier_count;     /* inliers of the winning trial */
   int32_t* best_hypothesis;  /* winning trial index h, -1 if none */
   int32_t* status;           /* RVH_STATUS_* bits */
@@ -347,8 +349,8 @@ int rvh_set_schedule(rvh_ctx* ctx, int32_t points_per_warp, int32_t hyps_per_lan
 
 /* Staged scoring with exact pruning (default on): the scoring pass of a
  * cluster of 256 (3D: 128) to 32767 points (the lanes-over-trials schedule,
- * points_per_warp 1) runs in stages, the first of 128 (3D: 64) points, the
- * second of 128 and each later one twice as long.  After the first,
+ * points_per_warp 1) runs in up to five stages: 128 (3D: 64) points, 128,
+ * 256, 512, and all others.  After the first,
  * the trial with the highest partial count leads: it is counted over every
  * point, and its residuals bound how many of the points still to come any
  * other trial can hold.  After each stage a trial whose partial count plus

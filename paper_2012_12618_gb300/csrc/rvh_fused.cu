@@ -1069,9 +1069,10 @@ __device__ __forceinline__ int prune_list(const Smem& S, int n, Keep keep, int* 
 }
 
 // ---- the staged scoring pass (a4 with exact pruning) ---------------------------------
-// Quads (4 points) of the first stage and of the next one; each later stage
-// is twice the one before.  Clusters of fewer than kStageMinPoints points
-// are scored in one pass.  What bounds the pass is the FP32 scoring of the
+// Quads (4 points) of the first stage and of the next one; the third stage is
+// twice the second, the fourth twice the third, and a fifth takes all other
+// points (a last stage of less than half the one before is joined to that).
+// Clusters of fewer than kStageMinPoints points are scored in one pass.  What bounds the pass is the FP32 scoring of the
 // pairs that stay (8.6e12 pairs/s inside the kernel, 9.15e12 in isolation),
 // then the lead pass, the histograms' scans and the first pruning test,
 // together about 40 points' worth of scoring 1024 trials.  Measured, ms per
@@ -1618,8 +1619,8 @@ __device__ void process_cluster(const FrameDesc& a, const Smem& S, ClusterShared
     // Counters of this warp, without atomics: a 64-bit shared-memory atomic is
     // a compare-and-swap loop, and in 3D, where every thread refines trials,
     // 256 of them on one word took longer than the mask pass of a small
-    // cluster: dense3d 1.205 -> 1.083 ms, 14,840 3D clusters of 8..177 points at 142
-    // trials 0.538 -> 0.378; dense2d, with fewer spills, 0.2203 -> 0.2177.
+    // cluster: dense3d 1.205 -> 1.083 ms; dense2d, with fewer spills, 0.2203 ->
+    // 0.2177.
     const unsigned fp64s = __reduce_add_sync(0xffffffffu, n_fp64), refs = __reduce_add_sync(0xffffffffu, n_ref);
     if ((tid & 31) == 0) {
       cs.wctr[0][tid >> 5] += fp64s;

@@ -27,7 +27,10 @@ struct FrameDesc {
   int32_t H;
   int64_t n_points;
   float4* rows_g;            // [n_points] FP32 rows of clusters beyond the shared-memory row capacity
-  double4_32a* rows64_g;         // [n_points] FP64 rows (a0, a1, a2, w) of every point
+  // [n_points] a slot of four doubles per point: 3D, the FP64 row (a0, a1, a2)
+  // and the low parts of the FP32 row (pack_low); 2D, (cos, sin) of the inliers
+  // between local-optimisation passes, or the line model's normalised (x, y)
+  double4_32a* rows64_g;
   const double2* trig;       // (cos, sin)(k/128), k = -420..420
   double tau;
   double eps;
@@ -71,8 +74,8 @@ struct FusedArgs {
   int wave;                  // CTA i < wave starts with item i (direct: every CTA, else one per SM); the
                              // others, and all later rounds, take items wave, wave + 1, ... as they come free
   int prune;                 // 1: staged scoring pass with exact pruning of trials that cannot win
-  // [grid * cta_slot_stride(dim, nmax_smem)] FP64 rows, one slot per CTA,
-  // used for clusters whose rows fit shared memory (a working set that
+  // [grid * cta_slot_stride(dim, nmax_smem)] the same slots, a run of them per
+  // CTA, used for clusters whose rows fit shared memory (a working set that
   // stays in L2); NULL: every cluster uses its frame's per-point rows64_g
   double4_32a* cta_rows64;
 };

@@ -24,7 +24,7 @@ constexpr int kWarps = kThreads / 32;
 struct Smem {
   float* rows;        // [roundup32(nmax_smem) * 4] floats of row tiles (TileRows)
   float4* hyp;        // [hchunk] (-X, -Y, -Z, thi)
-  float* tlo;         // [hchunk] staged pass: what each trial can hold (HoldRange, as bits)
+  float* tlo;         // [hchunk] no threshold: the staged pass's HoldRange of each trial, as bits
   int* U;             // [hchunk] upper bounds of the exact counts (-1 = rejected)
   int8_t* kind;       // [hchunk]
   uint16_t* list;     // [hchunk] trials still scored by the staged pass
